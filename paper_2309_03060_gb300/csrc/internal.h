@@ -84,6 +84,7 @@ struct Ctx {
   int* tc_err_host = nullptr;  // pinned copy of the tensor-core timeout flag
   cudaEvent_t tc_err_ev = nullptr;
   bool tc_err_pending = false;  // a copy of the flag is in flight
+  bool f64_tc_used = false;     // an FP64 tensor-core product ran since the last check
   int64_t tc_stall_ns = 0;      // armed by cola_test_stall_next_launch, consumed once
   void* host_pinned(size_t bytes);
   void count_launch() {
@@ -317,6 +318,14 @@ void check_cg_args(const cola_linop* op, const cola_cg_opts* o, int64_t R);
 // Raises COLA_ERR_TIMEOUT when a tensor-core kernel gave up waiting (and clears the flag).
 void tc_check_error(Ctx* c);        // synchronises the stream
 void tc_check_error_async(Ctx* c);  // reports an earlier call's timeout, queues a check
+void tc_check_earlier(Ctx* c, cudaStream_t user);  // FP64 products of earlier calls
+int* tc_errflag(Ctx* c);            // device flag the tensor-core kernels raise
+// FP64 mode step Y[r][m][i] = alpha sum_j F[i f_i + j f_j] X[r][j][m] + beta Y for
+// m < rest, i < n_out, j < n_in on the tensor cores (kron_f64.cu); false (nothing
+// launched) when the factor is too large for its digit images.
+bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, const double* X,
+                      int64_t size_in, const double* F, int64_t f_i, int64_t f_j, double beta,
+                      double* Y, int64_t size_out, int64_t R);
 // Fused MIXED CG MVM for Sum(Kron, Diag); see kron_tc.cu.  0 = not applicable.
 // p_new = z + beta p_old is formed in the first mode step (p_new != p_old).
 // rev: the first mode step walks its tiles in reverse order (and the slab

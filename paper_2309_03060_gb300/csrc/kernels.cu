@@ -3,7 +3,10 @@
 // tau_A N_B + N_A tau_B), the Kronecker-sum tridiagonal stencil, diagonal and
 // low-rank terms, deterministic per-vector reductions, leaf-gradient
 // contractions (App. B.2) and the SplitMix64 probe generator.
+#include <limits.h>
+
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "internal.h"
@@ -1089,6 +1092,22 @@ __global__ void k_add_partials(const T* P, T* G, int64_t count, int64_t nparts, 
 
 // =================================================================== hosts
 
+// Whether an FP64 mode step runs as digit products on the tensor cores
+// (kron_f64.cu) or on the FP64 units: the smaller of two times in us, fitted to
+// both kernels on factor sides 16 .. 1000 and 1 .. 4096 vectors (within 20 %):
+// 12 us for the digit images and a pipeline's fill plus 10.5 us per step (64
+// vectors x 128 outputs x 128 k) a CTA runs one after the other, against 6 us
+// plus 0.55e6 multiply-adds per us in 32 x 32 tiles.  Measured, us a step: 128^3 x
+// 16 264 against 6970; 64^2 x 64 21 against 37; 128^2 x 4 23 against 20.
+static bool f64_tc_pays(const Ctx* c, int64_t M, int64_t N, int64_t K, int64_t batch) {
+  const double tiles = (double)((M + 63) / 64) * (double)((N + 127) / 128) * (double)batch;
+  const double waves = std::ceil(tiles / c->num_sms);
+  const double tc = 12.0 + 10.5 * waves * (double)((K + 127) / 128);
+  const double fma = (double)((M + 31) / 32 * 32) * (double)((N + 31) / 32 * 32) * (double)K *
+                     (double)batch;
+  return tc < 6.0 + fma / 0.55e6;
+}
+
 template <typename T>
 void gemm(Ctx* c, int64_t M, int64_t N, int64_t K, double alpha, const T* A, int64_t lda_m,
           int64_t lda_k, int64_t sA, const T* B, int64_t ldb_k, int64_t ldb_n, int64_t sB,
@@ -1103,10 +1122,18 @@ void gemm(Ctx* c, int64_t M, int64_t N, int64_t K, double alpha, const T* A, int
                         ldc_n == 1 && M % 4 == 0 && N % 4 == 0 && lda_k % 4 == 0 &&
                         ldb_n % 4 == 0 && ldc_m % 4 == 0 && sA % 4 == 0 && sB % 4 == 0 &&
                         sC % 4 == 0 && a16(A) && a16(B) && a16(C);
-  // a product that fills fewer than a quarter of the SMs with 128 x 128 tiles
-  // runs one output per thread instead
   const int64_t tiles = (M + 127) / 128 * gy * batch;
   const int64_t total = M * N * batch;
+  // the FP64 mode steps of the Kronecker products: X [k][m] m-fast, C n-fast,
+  // one factor for the whole batch
+  if constexpr (std::is_same<T, double>::value) {
+    if (lda_m == 1 && lda_k == M && ldc_n == 1 && ldc_m == N && sB == 0 && N <= INT_MAX / 2 &&
+        K <= INT_MAX / 2 && f64_tc_pays(c, M, N, K, batch) &&
+        f64_tc_mode_step(c, M, (int)N, (int)K, alpha, A, sA, B, ldb_n, ldb_k, beta, C, sC, batch))
+      return;
+  }
+  // a product that fills fewer than a quarter of the SMs with 128 x 128 tiles
+  // runs one output per thread instead
   if (tiles * 4 < c->num_sms && total <= ((int64_t)1 << 24)) {
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 65535);
     k_gemm_small<T><<<grid, 256, 0, c->s>>>(g, total);

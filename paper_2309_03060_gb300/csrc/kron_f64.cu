@@ -1,0 +1,670 @@
+// FP64 Kronecker mode products on the tcgen05 tensor cores (sm_103a).
+//
+// One FP64 mode step  Y[r][m][i] = alpha sum_j F[i][j] X[r][j][m] + beta Y
+// (Sec. 3.2, Table 3) by an error-free split into integer digits, the scheme
+// of Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59, 2012; on tensor cores
+// Mukunoki et al. 2020): over a k chunk of at most 128 entries every factor
+// row and every vector gets a power-of-two scale from its largest exponent,
+//   f_ij = 2^(Ef_i - 55) sum_t a_t 256^(6-t),   x_jm = 2^(Ex_m - 54) sum_t b_t 256^(6-t),
+// with signed base-256 digits (|a_0| <= 256, |b_0| <= 128, the others in
+// [-128, 127]) that are exact in FP16.  The sums D_d = sum_{s+t=d} sum_j a_s b_t
+// of the 28 digit pairs with s + t <= 6 stay within 2^22 + d 2^21 <= 2^24 for 128
+// terms, so the FP32 accumulators hold them exactly; they are combined in 64-bit
+// integers (in units of D_5) and rounded to FP64 once.  What is lost: entries below 2^-55 of their row's or
+// vector's largest and the pairs s + t >= 7.
+//
+// Why: this GPU's FP64 units do 2 multiply-adds per clock and SM (1.2 TFLOP/s),
+// its tensor cores ~1900 TFLOP/s in FP16, so 28 products are still ~50 times
+// cheaper.  Every FP64 pipe use in the inner path is avoided: exponents and
+// digits come from integer operations, and so do the combination and its
+// conversion; only alpha, beta other than 1, 0 take FP64 instructions.
+//
+// Kernel layout (persistent, one 576-thread CTA per SM), tile = 64 vectors m x
+// 128 outputs i, step = tile x k chunk:
+//   warps 0-7   converters: load the 64 x 128 FP64 block into registers, find each
+//               vector's exponent and write the 7 digit images of the B operand
+//               (vectors x k, K-major, 128-byte swizzle, 112 KB)
+//   warps 8-15  drainers: add the accumulators up in 64-bit integers, scale, store
+//   warp 16     copies the factor's digit images (32 KB each, three buffers,
+//               cp.async.bulk from the prepared image, L2 resident)
+//   warp 17     issues the MMAs: factor digit s = 0 .. 6 outermost, so that group
+//               s is the last to use B digit 6 - s and completes accumulator D_s;
+//               D_s is drained and digit 6 - s refilled for the next step while
+//               the later groups run, and only D_6 and digit 0 are left when the
+//               MMAs of a step end
+// Measured (128^3 x 16, one mode step, 268 MB in and out): 264 us against 6.97 ms
+// on the FP64 units.  What bounds it: the integer work of converting 8192
+// entries and combining 8192 outputs per step (the ALU pipe), with the MMAs (224
+// of 128 x 64 x 16 per step, 48 clocks each by their shared-memory reads) at
+// 0.7 of the time; converting and draining in separate warps, both beside the
+// MMAs, took it from 395 us, no FP64-pipe instruction per output from 450 us, and
+// issuing from a converged warp (uniform descriptors) from 520 us.
+// Accumulators: D_0 .. D_6, 64 FP32 columns each of tensor memory.  Every
+// mbarrier wait gives up after ~2 s and raises the error flag.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "internal.h"
+#include "tc_ptx.cuh"
+
+namespace cola {
+
+namespace {
+
+constexpr int kDg = 7;             // digits per operand
+constexpr int kVec = 64;           // vectors per tile (N of the MMA)
+constexpr int kOut = 128;          // outputs per tile (M of the MMA)
+constexpr int kKc = 128;           // k chunk
+constexpr int kConvWarps = 8, kDrainWarps = 8;
+constexpr int kLoadWarp = kConvWarps + kDrainWarps, kMmaWarp = kLoadWarp + 1;
+constexpr int kThreadsF64 = 32 * (kMmaWarp + 1);
+constexpr uint32_t kBDig = kVec * kKc * 2;   // 16 KB per B digit
+constexpr uint32_t kADig = kOut * kKc * 2;   // 32 KB per A digit
+constexpr int kABufs = 3;
+constexpr size_t kSmemF64 = 1024 + kDg * kBDig + kABufs * kADig + 6144;
+constexpr int kPlain = 1 << 20;  // exponent mark of a factor row that takes plain products
+
+struct F64Params {
+  const double* X;
+  double* Y;
+  const double* F;      // the factor itself (plain products)
+  const uint16_t* img;  // [nchunks][kchunks][digit][k block][128][64], swizzled rows
+  const int* fexp;      // [nchunks][kchunks][128]
+  int64_t f_i, f_j;     // element strides of F
+  int64_t size_in, size_out;
+  int rest, tiles_m, ntiles, n_in, n_out, nchunks, kchunks;
+  double alpha, beta;
+  int has_alpha, has_beta;  // alpha != 1, beta != 0 (a compare is an FP64-pipe instruction)
+  int* err;
+  uint64_t stall_ns;
+};
+
+// Magnitude key of FP64 entries: the largest high word without the sign, or 1
+// when only low words are not zero, so that it is 0 only for +-0.
+__device__ __forceinline__ void mag_key(unsigned long long x, uint32_t& hi, uint32_t& lo) {
+  hi = max(hi, (uint32_t)(x >> 32) & 0x7fffffffu);
+  lo |= (uint32_t)x;
+}
+
+// A row or vector whose largest key is `key` has digits when it is zero or its
+// largest entry is finite and at least 2^-959 (below that a denormal entry
+// could still reach the digits, which fixed_digits does not expect); others
+// take plain FP64 products.
+__device__ __forceinline__ bool has_digits(int key) {
+  const int f = key >> 20;
+  return key == 0 || (f > 63 && f < 0x7ff);
+}
+
+constexpr unsigned long long kZeroDigits = 0x0100808080808080ull;
+
+// The digits of x, |x| < 2^(emax - 1022), scaled by 2^(52 + UP - (emax - 1023)) and rounded to
+// an integer v: v plus 128 in each byte 0 .. 5 and 256 at bit 48, so that bytes
+// 0 .. 5 are digits 6 .. 1 plus 128 and the bits from 48 on digit 0 plus 256.
+// emax > 63 (any value when x = 0): a zero or denormal entry shifts out
+// completely.
+template <int UP>
+__device__ __forceinline__ unsigned long long fixed_digits(unsigned long long x, int emax) {
+  const uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
+  const int sh = min(63, emax - (int)((hi >> 20) & 0x7ffu));
+  const unsigned long long m =
+      (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << (UP + 1);
+  const unsigned long long w = m >> sh;  // twice |v|, one bit below it
+  const long long sg = (int)hi >> 31;    // 0 or -1
+  constexpr long long bias = (long long)kZeroDigits;
+  // x >= 0: floor((w + 1) / 2); x < 0: floor(-w / 2), as ~w + 1 = -w; plus the bias
+  return (unsigned long long)(((long long)(w ^ (unsigned long long)sg) + (2 * bias + 1)) >> 1);
+}
+// Digit t of two values as an FP16 pair: 0x6400 | b is 1024 + b for b < 1024,
+// the bias comes off exactly.
+template <int t>
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
+  constexpr int byte = 6 - t;  // byte position in the 64-bit word
+  const uint32_t aw = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32);
+  const uint32_t bw = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
+  constexpr uint32_t p = byte & 3;
+  uint32_t w, bias;
+  if constexpr (t == 0) {
+    w = __byte_perm(aw, bw, 0x7632) | 0x64006400u;
+    bias = 0x65006500u;  // 1024 + 256
+  } else {
+    w = (__byte_perm(aw, bw, p | (p << 4) | ((4 + p) << 8) | ((4 + p) << 12)) & 0x00ff00ffu) |
+        0x64006400u;
+    bias = 0x64806480u;  // 1024 + 128
+  }
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w),
+                            *reinterpret_cast<const __half2*>(&bias));
+  return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+// a 2^e for an e outside the range of scaled_double (overflow, denormals).
+__device__ __noinline__ double far_scale(long long a, int e) {
+  return ldexp(__ll2double_rn(a), e);
+}
+
+// a 2^e rounded to FP64 for 1023 + 62 + |e| within the exponent range, by
+// integer operations (an FP64 conversion is two instructions of 16 clocks each
+// on the SM's FP64 units): the leading bit of |a| goes to bit 63, bits 63 .. 11
+// rounded are the significand with its hidden bit, which adds 1 to the exponent.
+__device__ __forceinline__ double scaled_double(long long a, int e) {
+  const uint32_t sg = (uint32_t)(a >> 63);
+  const unsigned long long m = ((unsigned long long)a ^ (unsigned long long)(long long)(int)sg) -
+                               (unsigned long long)(long long)(int)sg;
+  const int lz = __clzll((long long)m);  // 64 for 0: the shift below leaves 0
+  const unsigned long long n = lz < 64 ? m << lz : 0ull;
+  const unsigned long long r = (n + 0x400ull) >> 11;
+  const bool carry = n + 0x400ull < n;  // rounded up to 2^64
+  uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(1023 + 62 - lz + e) << 20);
+  if (carry) hi = (uint32_t)(1023 + 64 - lz + e) << 20;
+  if (m == 0) hi = 0;
+  return __hiloint2double((int)(hi | (sg & 0x80000000u)), (int)(uint32_t)r);
+}
+constexpr int kFarExp = 450;  // |exponent| of a row or vector up to which it does
+
+// The dot product of one output whose factor row or vector has no digits.
+__device__ __noinline__ double plain_dot(const double* f, int64_t f_j, const double* x,
+                                         int64_t rest, int k0, int k1) {
+  double v = 0.0;
+  for (int k = k0; k < k1; ++k) v = fma(f[k * f_j], x[(int64_t)k * rest], v);
+  return v;
+}
+
+// The digit images and exponents of one factor (chunk): block (row of the
+// padded 128-row output chunk, output chunk, k chunk), one thread per k.
+__global__ void __launch_bounds__(kKc) k_f64_digits(const double* F, int64_t f_i, int64_t f_j,
+                                                    int n_out, int n_in, int kchunks,
+                                                    uint16_t* img, int* fexp) {
+  const int row = blockIdx.x, nc = blockIdx.y, kc = blockIdx.z, k = threadIdx.x;
+  const int i = nc * kOut + row, j = kc * kKc + k;
+  __shared__ int smax[kKc / 32];
+  const double x = (i < n_out && j < n_in) ? F[i * f_i + j * f_j] : 0.0;
+  uint32_t xh = 0, xl = 0;
+  mag_key((unsigned long long)__double_as_longlong(x), xh, xl);
+  int mx = xh | (xh == 0 && xl != 0 ? 1 : 0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((k & 31) == 0) smax[k >> 5] = mx;
+  __syncthreads();
+  mx = max(max(smax[0], smax[1]), max(smax[2], smax[3]));
+  const int emax = mx >> 20;
+  const bool dig = has_digits(mx);
+  const int64_t blk = (int64_t)nc * kchunks + kc;
+  if (k == 0) fexp[blk * kOut + row] = dig ? emax - 1023 : kPlain;
+  const unsigned long long u =
+      dig && mx ? fixed_digits<3>((unsigned long long)__double_as_longlong(x), emax) : kZeroDigits;
+  // digit t: k block (k / 64), row, 16-byte chunk (k / 8) mod 8 swizzled by the row
+  uint16_t* p = img + blk * (kDg * kADig / 2) + (size_t)(k >> 6) * (kOut * 64) + row * 64 +
+                ((((k >> 3) & 7) ^ (row & 7)) << 3) + (k & 7);
+  constexpr size_t st = kADig / 2;
+  p[0 * st] = (uint16_t)digit_pair<0>(u, u);
+  p[1 * st] = (uint16_t)digit_pair<1>(u, u);
+  p[2 * st] = (uint16_t)digit_pair<2>(u, u);
+  p[3 * st] = (uint16_t)digit_pair<3>(u, u);
+  p[4 * st] = (uint16_t)digit_pair<4>(u, u);
+  p[5 * st] = (uint16_t)digit_pair<5>(u, u);
+  p[6 * st] = (uint16_t)digit_pair<6>(u, u);
+}
+
+// One (tile, k chunk) step.
+struct F64Step {
+  int r, m0, nc, kc;
+};
+__device__ __forceinline__ F64Step step_of(const F64Params& p, int tile, int kc) {
+  F64Step s;
+  s.nc = tile % p.nchunks;
+  const int t = tile / p.nchunks;
+  s.r = t / p.tiles_m;
+  s.m0 = (t - s.r * p.tiles_m) * kVec;
+  s.kc = kc;
+  return s;
+}
+
+__device__ __forceinline__ void mad_wide(long long& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+
+// Folds accumulator D_T's 32 columns into the integer sums (units of D_5).
+template <int T>
+__device__ __forceinline__ void fold(uint32_t taddr, long long (&acc)[32]) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    uint32_t v[8];
+    tmem_ld8(taddr + T * kVec + h * 8, v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int c = h * 8 + e;
+      const int d = __float2int_rn(__uint_as_float(v[e]));
+      if constexpr (T == 0) {
+        acc[c] = (long long)((unsigned long long)((uint32_t)d << 8) << 32);
+      } else if constexpr (T == 1) {
+        acc[c] += (long long)((unsigned long long)(uint32_t)d << 32);
+      } else if constexpr (T == 6) {
+        mad_wide(acc[c], (d + 128) >> 8, 1);
+      } else {
+        mad_wide(acc[c], d, 1 << (8 * (5 - T)));
+      }
+    }
+  }
+}
+
+// Writes digit T of this thread's four 8-entry k runs (run h at k = 8 oct + 32 h:
+// k block h / 2, 16-byte chunk (oct + 4 h) mod 8).
+template <int T>
+__device__ __forceinline__ void put_digit(unsigned char* bdig, const unsigned long long (&u)[32],
+                                          int n, int oct, int kpad) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    if (oct * 8 + h * 32 >= kpad) continue;
+    uint4 w;
+    w.x = digit_pair<T>(u[8 * h + 0], u[8 * h + 1]);
+    w.y = digit_pair<T>(u[8 * h + 2], u[8 * h + 3]);
+    w.z = digit_pair<T>(u[8 * h + 4], u[8 * h + 5]);
+    w.w = digit_pair<T>(u[8 * h + 6], u[8 * h + 7]);
+    const int ch = (oct + 4 * (h & 1)) ^ (n & 7);
+    *reinterpret_cast<uint4*>(bdig + T * kBDig + (h >> 1) * (kBDig / 2) + n * 128 + ch * 16) = w;
+  }
+}
+
+// The MMAs of factor digit a with every B digit t <= 6 - a (t downwards: digit
+// 0 is refilled last).  One warp issues 224 MMAs per step, so the k loop is
+// unrolled with constant descriptor offsets.
+template <bool FULL>
+__device__ __forceinline__ void issue_group(uint32_t tmem, uint64_t ad, uint64_t bdesc,
+                                            uint32_t idesc, int a, int ksteps,
+                                            uint32_t elect) {
+#pragma unroll 1
+  for (int t = kDg - 1 - a; t >= 0; --t) {
+    const uint32_t d = tmem + (uint32_t)(a + t) * kVec;
+    const uint64_t bd = bdesc + (uint64_t)((uint32_t)t * (kBDig >> 4));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (!FULL && k >= ksteps) break;
+      const uint64_t ko = (uint64_t)(k & 3) * 2;
+      mma_f16_one(d, ad + (uint64_t)(k >> 2) * (kADig >> 5) + ko,
+                   bd + (uint64_t)(k >> 2) * (kBDig >> 5) + ko, idesc,
+                   k == 0 ? (a == 0 ? 0u : 1u) : 1u, elect);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreadsF64, 1)
+    k_kron_f64_tc(const __grid_constant__ F64Params p) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  unsigned char* bdig = base;
+  unsigned char* adig = base + kDg * kBDig;
+  uint64_t* afull = (uint64_t*)(adig + kABufs * kADig);
+  uint64_t* aempty = afull + kABufs;
+  uint64_t* ready = aempty + kABufs;  // B digits written, D of the step before drained
+  uint64_t* dfull = ready + 1;        // [7] D_s complete, B digit 6 - s no longer read
+  uint64_t* kfull = dfull + kDg;      // [2] keys of an even / odd step written
+  uint64_t* kfree = kfull + 2;        // [2] and no longer read
+  uint64_t* drain = kfree + 2;
+  uint64_t* stall = drain + 1;  // never completed (time-out test)
+  uint32_t* tmem_slot = (uint32_t*)(stall + 1);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  // per (step parity, converter k group, vector): largest magnitude key; then
+  // per (parity, vector): the key, and per (parity, warp) whether any vector of
+  // the step needs more than the exponent addition
+  int* cmax = (int*)(tmem_slot + 2);     // [2][4][64]
+  int* ckey = cmax + 8 * kVec;           // [2][64]
+  volatile int* cfar = ckey + 2 * kVec;  // [2][2]
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < kABufs; ++s) {
+      mbar_init(&afull[s], 1);
+      mbar_init(&aempty[s], 1);
+    }
+    mbar_init(ready, kConvWarps + kDrainWarps);
+    for (int t = 0; t < kDg; ++t) mbar_init(&dfull[t], 1);
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&kfull[q], kConvWarps);
+      mbar_init(&kfree[q], kDrainWarps);
+    }
+    mbar_init(drain, 1);
+    mbar_init(stall, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const int mine = (p.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int nsteps = (int)blockIdx.x < p.ntiles ? mine * p.kchunks : 0;
+  const int kb_last = (p.n_in - (p.kchunks - 1) * kKc + 63) / 64;  // k blocks, last chunk
+
+  if (warp == kLoadWarp) {
+    // -------------------------------------------------- factor digit copies
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0, issued = 0, issued_ph = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x) {
+        const int nc = tile % p.nchunks;
+        for (int kc = 0; kc < p.kchunks && ok; ++kc) {
+          const uint32_t bytes = (kc == p.kchunks - 1 ? kb_last : 2) * (kADig / 2);
+          const unsigned char* src = (const unsigned char*)p.img +
+                                     ((int64_t)nc * p.kchunks + kc) * (int64_t)(kDg * kADig);
+          for (int a = 0; a < kDg; ++a) {
+            if (!mbar_wait(&aempty[s], ph ^ 1u, abort_flag, p.err)) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_expect_tx(&afull[s], bytes);
+            bulk_g2s(adig + s * kADig, src + a * kADig, bytes, &afull[s]);
+            issued |= 1u << s;
+            issued_ph = (issued_ph & ~(1u << s)) | (ph << s);
+            if (++s == kABufs) {
+              s = 0;
+              ph ^= 1u;
+            }
+          }
+        }
+      }
+      // the latest copy into each buffer is the only one that can be in flight
+      for (int b = 0; b < kABufs; ++b)
+        if (issued & (1u << b)) mbar_wait_own(&afull[b], (issued_ph >> b) & 1u, p.err);
+    }
+    __syncwarp();
+  } else if (warp == kMmaWarp) {
+    // ------------------------------------------------------------------ MMA
+    // the whole warp runs the loop, one elected lane issues
+    const uint32_t elect = elect_one();
+    constexpr uint32_t idesc = idesc_f16(kOut, kVec);
+    bool ok = true;
+    if (p.stall_ns)
+      ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns));
+    const uint64_t adesc = sw128_desc(smem_u32(adig)), bdesc = sw128_desc(smem_u32(bdig));
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
+    int s = 0;
+    uint32_t ph = 0, sph = 0;
+    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x) {
+      for (int kc = 0; kc < p.kchunks && ok; ++kc, sph ^= 1u) {
+        const int kleft = p.n_in - kc * kKc;
+        const int ksteps = kleft >= kKc ? 8 : (kleft + 15) / 16;
+        ok = __all_sync(0xffffffffu, mbar_wait(ready, sph, abort_flag, p.err));
+        if (!ok) break;
+        tc_fence_after();
+        for (int a = 0; a < kDg; ++a) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&afull[s], ph, abort_flag, p.err));
+          if (!ok) break;
+          tc_fence_after();
+          // descriptors advance by address / 16: 2 per 16-wide k step
+          const uint64_t ad = adesc + (uint64_t)((uint32_t)s * (kADig >> 4));
+          if (ksteps == 8)
+            issue_group<true>(tmem, ad, bdesc, idesc, a, 8, elect);
+          else
+            issue_group<false>(tmem, ad, bdesc, idesc, a, ksteps, elect);
+          mma_commit_one(&dfull[a], elect);
+          mma_commit_one(&aempty[s], elect);
+          if (++s == kABufs) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+    }
+    // the elected lane's commit covers every MMA it issued
+    mma_commit_one(drain, elect);
+    if (elect) mbar_wait_own(drain, 0, p.err);
+    __syncwarp();
+  } else if (warp < kConvWarps) {
+    // ----------------------------------------------------------- converters
+    // vector n of the tile, 8-entry k runs at k = 8 oct + 32 h, h < 4
+    const int n = (warp & 1) * 32 + lane, oct = warp >> 1;
+    unsigned long long u[32];
+    auto load = [&](const F64Step& s) {
+      const int m = s.m0 + n;
+      const double* x = p.X + s.r * p.size_in + m;
+      const int k0 = s.kc * kKc + oct * 8;
+      if (m < p.rest && k0 + 104 <= p.n_in) {
+        x += (int64_t)k0 * p.rest;
+#pragma unroll
+        for (int e = 0; e < 32; ++e)
+          u[e] = (unsigned long long)__double_as_longlong(
+              __ldg(x + ((e & 7) + (e >> 3) * 32) * p.rest));
+        return;
+      }
+#pragma unroll
+      for (int e = 0; e < 32; ++e) {
+        const int k = k0 + (e & 7) + (e >> 3) * 32;
+        u[e] = (m < p.rest && k < p.n_in)
+                   ? (unsigned long long)__double_as_longlong(x[k * p.rest])
+                   : 0ull;
+      }
+    };
+    int tile = blockIdx.x, kc = 0;
+    if (nsteps > 0) load(step_of(p, tile, 0));
+    bool ok = true;
+    for (int st = 0; st < nsteps; ++st) {
+      const int par = st & 1;
+      uint32_t xh = 0, xl = 0;
+#pragma unroll
+      for (int e = 0; e < 32; ++e) mag_key(u[e], xh, xl);
+      cmax[(par * 4 + oct) * kVec + n] = (int)(xh | (xh == 0 && xl != 0 ? 1u : 0u));
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      int key = 0;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) key = max(key, cmax[(par * 4 + o) * kVec + n]);
+      const int emax = key >> 20;
+      const bool dig = key != 0 && has_digits(key);
+      if (st > 1) {  // the drainers are done with the keys of step st - 2
+        if (ok) ok = mbar_wait(&kfree[par], (uint32_t)((st >> 1) + 1) & 1u, abort_flag, p.err);
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      if (oct == 0) {
+        ckey[par * kVec + n] = key;
+        const bool far = key != 0 && (!dig || abs(emax - 1023) > kFarExp);
+        const bool any = __any_sync(0xffffffffu, far);
+        if (lane == 0) cfar[par * 2 + warp] = any;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&kfull[par]);
+#pragma unroll
+      for (int e = 0; e < 32; ++e) u[e] = dig ? fixed_digits<2>(u[e], emax) : kZeroDigits;
+        // keep the conversion ahead of the waits below, beside the MMAs
+#pragma unroll
+      for (int e = 0; e < 32; ++e) asm volatile("" : "+l"(u[e]));
+      const int kpad = (min(p.n_in - kc * kKc, kKc) + 15) / 16 * 16;
+      // digit 6 - S is free once MMA group S of the step before is done
+      const uint32_t dph = (uint32_t)((st + 1) & 1);
+#define COLA_DIGIT(S)                                                      \
+  if (st > 0) {                                                            \
+    if (ok) ok = mbar_wait(&dfull[S], dph, abort_flag, p.err);             \
+    ok = __all_sync(0xffffffffu, ok);                                      \
+  }                                                                        \
+  put_digit<6 - S>(bdig, u, n, oct, kpad);
+      COLA_DIGIT(0)
+      COLA_DIGIT(1)
+      COLA_DIGIT(2)
+      COLA_DIGIT(3)
+      COLA_DIGIT(4)
+      COLA_DIGIT(5)
+      COLA_DIGIT(6)
+#undef COLA_DIGIT
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ready);
+      if (++kc == p.kchunks) {
+        kc = 0;
+        tile += gridDim.x;
+      }
+      if (st + 1 < nsteps) load(step_of(p, tile, kc));
+      if (st + 2 < nsteps) {  // the block after it: DRAM to L2, two 128-byte lines a thread
+        const bool wrap = kc + 1 == p.kchunks;
+        const F64Step f = step_of(p, wrap ? tile + (int)gridDim.x : tile, wrap ? 0 : kc + 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int k = f.kc * kKc + (tid >> 2) + 64 * h, m = f.m0 + (tid & 3) * 16;
+          if (k < p.n_in && m < p.rest)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.X + f.r * p.size_in +
+                                                           (int64_t)k * p.rest + m));
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------- drainers
+    // output lane 32 (warp mod 4) + lane, 32 vectors from oc0
+    const int orow = (warp & 3) * 32 + lane, oc0 = ((warp - kConvWarps) >> 2) * 32;
+    const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)oc0;
+    long long acc[32];
+    int tile = blockIdx.x, kc = 0;
+    bool ok = true;
+    if (nsteps > 0 && lane == 0) mbar_arrive(ready);  // nothing to drain before step 0
+    for (int st = 0; st < nsteps; ++st) {
+      const int par = st & 1;
+      const int nc = tile % p.nchunks;
+      // the factor row's exponent, ahead of its use in the store
+      const int ef = __ldg(&p.fexp[((int64_t)nc * p.kchunks + kc) * kOut + orow]);
+#define COLA_DIGIT(S)                                                      \
+  if (ok) ok = mbar_wait(&dfull[S], (uint32_t)par, abort_flag, p.err);     \
+  ok = __all_sync(0xffffffffu, ok);                                        \
+  tc_fence_after();                                                        \
+  if (ok) fold<S>(taddr, acc);
+      COLA_DIGIT(0)
+      COLA_DIGIT(1)
+      COLA_DIGIT(2)
+      COLA_DIGIT(3)
+      COLA_DIGIT(4)
+      COLA_DIGIT(5)
+      COLA_DIGIT(6)
+#undef COLA_DIGIT
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0 && st + 1 < nsteps) mbar_arrive(ready);
+      if (ok) ok = mbar_wait(&kfull[par], (uint32_t)(st >> 1) & 1u, abort_flag, p.err);
+      ok = __all_sync(0xffffffffu, ok);
+      const F64Step cur = step_of(p, tile, kc);
+      const int i = nc * kOut + orow;
+      const int cnt = min(32, p.rest - cur.m0 - oc0);
+      if (ok && i < p.n_out && cnt > 0) {
+        double* y = p.Y + cur.r * p.size_out + (int64_t)(cur.m0 + oc0) * p.n_out + i;
+        const int* keys = ckey + par * kVec + oc0;
+        const bool near = abs(ef) <= kFarExp && !(cfar[par * 2] | cfar[par * 2 + 1]);
+        const int e0 = ef - 53 - 1023;
+        // Y's old values join with beta (first k chunk) or 1 (later chunks)
+        const bool old = kc > 0 || p.has_beta;
+        const double bo = kc > 0 ? 1.0 : p.beta;
+        if (near && cnt == 32) {  // no branch per output
+#pragma unroll
+          for (int g = 0; g < 32; g += 4) {
+            double v[4];
+            if (old) {
+#pragma unroll
+              for (int c = 0; c < 4; ++c) v[c] = y[(g + c) * p.n_out];
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              double w = scaled_double(acc[g + c], e0 + (keys[g + c] >> 20));
+              if (p.has_alpha) w *= p.alpha;
+              if (old) w = fma(bo, v[c], w);
+              y[(g + c) * p.n_out] = w;
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < cnt; ++c) {
+            long long ac = 0;
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+              if (q == c) ac = acc[q];
+            const int key = keys[c];
+            double v;
+            if (near) {
+              v = scaled_double(ac, e0 + (key >> 20));
+            } else if (has_digits(key) && ef != kPlain) {
+              v = far_scale(ac, e0 + (key >> 20));
+            } else {
+              v = plain_dot(p.F + i * p.f_i, p.f_j, p.X + cur.r * p.size_in + cur.m0 + oc0 + c,
+                            p.rest, kc * kKc, min(p.n_in, (kc + 1) * kKc));
+            }
+            if (p.has_alpha) v *= p.alpha;
+            if (old) v = fma(bo, *y, v);
+            *y = v;
+            y += p.n_out;
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&kfree[par]);
+      if (++kc == p.kchunks) {
+        kc = 0;
+        tile += gridDim.x;
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(512)
+                 : "memory");
+  }
+}
+
+}  // namespace
+
+bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, const double* X,
+                      int64_t size_in, const double* F, int64_t f_i, int64_t f_j, double beta,
+                      double* Y, int64_t size_out, int64_t R) {
+  F64Params p{};
+  p.nchunks = (n_out + kOut - 1) / kOut;
+  p.kchunks = (n_in + kKc - 1) / kKc;
+  const int64_t tiles_m = (rest + kVec - 1) / kVec;
+  // indices within one vector block and tile numbers are 32-bit
+  if (rest * std::max(n_in, n_out) >= ((int64_t)1 << 31) - 1024 ||
+      R * tiles_m * p.nchunks * p.kchunks >= ((int64_t)1 << 31) - 1024)
+    return false;
+  p.tiles_m = (int)tiles_m;
+  p.ntiles = (int)(R * tiles_m * p.nchunks);
+  const size_t blocks = (size_t)p.nchunks * p.kchunks;
+  if (p.nchunks > 65535 || p.kchunks > 65535 || blocks > 1024) return false;
+  uint16_t* img = (uint16_t*)c->ws.get("f64.img", blocks * kDg * kADig);
+  int* fexp = (int*)c->ws.get("f64.exp", blocks * kOut * 4);
+  k_f64_digits<<<dim3(kOut, (unsigned)p.nchunks, (unsigned)p.kchunks), kKc, 0, c->s>>>(
+      F, f_i, f_j, n_out, n_in, p.kchunks, img, fexp);
+  c->count_launch();
+  p.X = X;
+  p.Y = Y;
+  p.F = F;
+  p.img = img;
+  p.fexp = fexp;
+  p.f_i = f_i;
+  p.f_j = f_j;
+  p.rest = (int)rest;
+  p.size_in = size_in;
+  p.size_out = size_out;
+  p.n_in = n_in;
+  p.n_out = n_out;
+  p.alpha = alpha;
+  p.beta = beta;
+  p.has_alpha = alpha != 1.0;
+  p.has_beta = beta != 0.0;
+  p.err = tc_errflag(c);
+  if (c->tc_stall_ns > 0 && !c->capturing) {
+    p.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
+    c->tc_stall_ns = 0;
+  }
+  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemF64));
+  const int grid = (int)std::min<int64_t>(p.ntiles, c->num_sms);
+  k_kron_f64_tc<<<grid, kThreadsF64, kSmemF64, c->s>>>(p);
+  c->count_launch();
+  c->f64_tc_used = true;
+  COLA_CUDA(cudaGetLastError());
+  return true;
+}
+
+}  // namespace cola

@@ -69,6 +69,7 @@ void* Ctx::host_pinned(size_t bytes) {
 // A caller that already works on the context's own stream needs no join.
 StreamJoin::StreamJoin(Ctx* c_, cola_stream s) : c(c_), user((cudaStream_t)s) {
   COLA_CUDA(cudaSetDevice(c->device));
+  tc_check_earlier(c, user);
   if (user == c->s) return;
   COLA_CUDA(cudaEventRecord(c->ev_a, user));
   COLA_CUDA(cudaStreamWaitEvent(c->s, c->ev_a, 0));

@@ -281,7 +281,7 @@ __device__ __forceinline__ void issue_group(uint32_t tmem, uint64_t ad, uint64_t
     for (int k = 0; k < 8; ++k) {
       if (!FULL && k >= ksteps) break;
       const uint64_t ko = (uint64_t)(k & 3) * 2;
-      mma_f16_one(d, ad + (uint64_t)(k >> 2) * (kADig >> 5) + ko,
+      mma_one(d, ad + (uint64_t)(k >> 2) * (kADig >> 5) + ko,
                    bd + (uint64_t)(k >> 2) * (kBDig >> 5) + ko, idesc,
                    k == 0 ? (a == 0 ? 0u : 1u) : 1u, elect);
     }
@@ -392,11 +392,11 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       for (int kc = 0; kc < p.kchunks && ok; ++kc, sph ^= 1u) {
         const int kleft = p.n_in - kc * kKc;
         const int ksteps = kleft >= kKc ? 8 : (kleft + 15) / 16;
-        ok = __all_sync(0xffffffffu, mbar_wait(ready, sph, abort_flag, p.err));
+        ok = mbar_wait_warp(ready, sph, abort_flag, p.err);
         if (!ok) break;
         tc_fence_after();
         for (int a = 0; a < kDg; ++a) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&afull[s], ph, abort_flag, p.err));
+          ok = mbar_wait_warp(&afull[s], ph, abort_flag, p.err);
           if (!ok) break;
           tc_fence_after();
           // descriptors advance by address / 16: 2 per 16-wide k step

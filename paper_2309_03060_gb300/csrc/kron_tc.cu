@@ -528,16 +528,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
       : "memory");
 }
 
-__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
-                                            uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 // 2-D tiled TMA load of the box at (x, y) of a tensor map into shared memory.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
                                             uint64_t* bar) {
@@ -813,28 +803,32 @@ __global__ void __launch_bounds__(kThreadsFs, 1) k_kron_tc_fs(const __grid_const
     }
   } else if (warp == kFsMmaWarp) {
     // ------------------------------------------------------------------- MMA
-    if (lane == 0) {
+    // the whole warp runs the loop, one elected lane issues
+    {
+      const uint32_t elect = elect_one();
+      const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);  // warp-uniform
       constexpr uint32_t idesc = idesc_bf16(kTileM, kTileM);  // M = outputs, N = rows
-      bool ok = mbar_wait(afac, 0, abort_flag, p.err);
-      if (ok && p.stall_ns) ok = mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns);
+      bool ok = mbar_wait_warp(afac, 0, abort_flag, p.err);
+      if (ok && p.stall_ns)
+        ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns));
       tc_fence_after();
       const uint32_t bbase = smem_u32(bsm);
       int sb = 0;
       uint32_t phb = 0;
       int64_t it = 0;
       for (int64_t t0 = blockIdx.x; t0 < p.ntiles && ok; t0 += gridDim.x, ++it) {
-        if (!mbar_wait(dempty, (uint32_t)(it & 1) ^ 1u, abort_flag, p.err)) break;
+        if (!mbar_wait_warp(dempty, (uint32_t)(it & 1) ^ 1u, abort_flag, p.err)) break;
         tc_fence_after();
         uint32_t acc_small = 0;
         for (int kb = 0; kb < p.kblocks; ++kb) {
-          if (!mbar_wait(&bfull[sb], phb, abort_flag, p.err)) {
+          if (!mbar_wait_warp(&bfull[sb], phb, abort_flag, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const int steps = (kb == p.kblocks - 1) ? p.ksteps_last : 4;
           const uint32_t bst = bbase + (uint32_t)sb * (uint32_t)TV * kFsBTermBytes;
-          const uint32_t fa = tmem_base + kFsFactorCol0 + (uint32_t)kb * 32u;
+          const uint32_t fa = tmem + kFsFactorCol0 + (uint32_t)kb * 32u;
           for (int kk = 0; kk < steps; ++kk) {
 #pragma unroll
             for (int ti = 0; ti < TF; ++ti)
@@ -845,24 +839,24 @@ __global__ void __launch_bounds__(kThreadsFs, 1) k_kron_tc_fs(const __grid_const
                 const uint64_t bd =
                     sw128_desc(bst + (uint32_t)tv * kFsBTermBytes + (uint32_t)kk * 32u);
                 if (ti == 0 && tv == 0) {
-                  mma_bf16_ta(tmem_base, a, bd, idesc, (kb | kk) ? 1u : 0u);
+                  mma_one_ta(tmem, a, bd, idesc, (kb | kk) ? 1u : 0u, elect);
                 } else {
-                  mma_bf16_ta(tmem_base + kFsSmallCol, a, bd, idesc, acc_small);
+                  mma_one_ta(tmem + kFsSmallCol, a, bd, idesc, acc_small, elect);
                   acc_small = 1;
                 }
               }
           }
-          mma_commit(&bempty[sb]);
+          mma_commit_one(&bempty[sb], elect);
           if (++sb == 2) {
             sb = 0;
             phb ^= 1u;
           }
         }
         if (!ok) break;
-        mma_commit(dfull);
+        mma_commit_one(dfull, elect);
       }
-      mma_commit(drain);
-      mbar_wait_own(drain, 0, p.err);
+      mma_commit_one(drain, elect);
+      if (elect) mbar_wait_own(drain, 0, p.err);
     }
     __syncwarp();
   } else {
@@ -1320,10 +1314,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------- MMA
-    if (lane == 0) {
+    // the whole warp runs the loop, one elected lane issues
+    {
+      const uint32_t elect = elect_one();
+      const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);  // warp-uniform
       constexpr uint32_t idesc = idesc_bf16(kTileM, kTileM);  // M = outputs, N = rows
       bool ok = true;
-      if (L.stall_ns) ok = mbar_wait_slow(stall, 0, abort_flag, L.err, L.stall_ns);
+      if (L.stall_ns)
+        ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, L.err, L.stall_ns));
       int s = 0;
       uint32_t ph = 0;
       int64_t it = 0;
@@ -1333,12 +1331,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         int64_t lt;
         const int kblocks = src.get(t, lt).kblocks;
         const int b = (int)(it & 1);
-        if (!mbar_wait(&aempty[b], (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, L.err)) break;
+        if (!mbar_wait_warp(&aempty[b], (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag, L.err)) break;
         tc_fence_after();
-        const uint32_t d_big = tmem_base + (uint32_t)b * 256u, d_small = d_big + 128u;
+        const uint32_t d_big = tmem + (uint32_t)b * 256u, d_small = d_big + 128u;
         uint32_t acc_big = 0, acc_small = 0;
         for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&full[s], ph, abort_flag, L.err)) {
+          if (!mbar_wait_warp(&full[s], ph, abort_flag, L.err)) {
             ok = false;
             break;
           }
@@ -1356,25 +1354,25 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const uint64_t bd =
                     sw128_desc(st + (uint32_t)tv * kGemmTermBytes + (uint32_t)kk * 32u);
                 if (ti == 0 && tv == 0) {
-                  mma_bf16(d_big, ad, bd, idesc, acc_big);
+                  mma_one(d_big, ad, bd, idesc, acc_big, elect);
                   acc_big = 1;
                 } else {
-                  mma_bf16(d_small, ad, bd, idesc, acc_small);
+                  mma_one(d_small, ad, bd, idesc, acc_small, elect);
                   acc_small = 1;
                 }
               }
           }
-          mma_commit(&empty[s]);
+          mma_commit_one(&empty[s], elect);
           if (++s == L.stages) {
             s = 0;
             ph ^= 1u;
           }
         }
         if (!ok) break;
-        mma_commit(&afull[b]);
+        mma_commit_one(&afull[b], elect);
       }
-      mma_commit(drain);
-      mbar_wait_own(drain, 0, L.err);
+      mma_commit_one(drain, elect);
+      if (elect) mbar_wait_own(drain, 0, L.err);
     }
     __syncwarp();
   } else {
@@ -1861,30 +1859,38 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
     if (ok && it > 0) drain_y(slab_at(blockIdx.x + (it - 1) * (int64_t)gridDim.x), it - 1);
   } else if (warp == kFsMmaWarp) {
     // ------------------------------------------------------------------- MMA
-    if (lane == 0) {
+    // the whole warp runs the loop, one elected lane issues
+    {
+      const uint32_t elect = elect_one();
+      const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);  // warp-uniform
       constexpr uint32_t idesc = idesc_bf16(kTileM, kSlabN);  // M = outputs, N = 128 rows
       // K3's split image: TF terms x 2 k blocks of 128 swizzled rows
-      mbar_arrive_expect_tx(a3full, (uint32_t)(TF * 2) * kFsBTermBytes);
+      if (elect) {
+        mbar_arrive_expect_tx(a3full, (uint32_t)(TF * 2) * kFsBTermBytes);
 #pragma unroll
-      for (int b = 0; b < TF * 2; ++b)
-        bulk_g2s(a3 + (size_t)b * kFsBTermBytes, p.img3 + (size_t)b * p.img_rows3 * kBlockK,
-                 kFsBTermBytes, a3full);
-      bool ok = mbar_wait_own(a3full, 0, p.err) && mbar_wait(afac, 0, abort_flag, p.err);
-      if (ok && p.stall_ns) ok = mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns);
+        for (int b = 0; b < TF * 2; ++b)
+          bulk_g2s(a3 + (size_t)b * kFsBTermBytes, p.img3 + (size_t)b * p.img_rows3 * kBlockK,
+                   kFsBTermBytes, a3full);
+      }
+      __syncwarp();
+      bool ok = __all_sync(0xffffffffu, mbar_wait_own(a3full, 0, p.err)) &&
+                mbar_wait_warp(afac, 0, abort_flag, p.err);
+      if (ok && p.stall_ns)
+        ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns));
       tc_fence_after();
       // operand descriptors: base descriptor plus (offset >> 4), the 14-bit
       // address field holding any shared-memory address below 256 KB
       const uint64_t bdesc0 = sw128_desc(smem_u32(bbuf)), adesc0 = sw128_desc(smem_u32(a3));
-      const uint32_t d_dom = tmem_base + kSlabAccCol, d_small = d_dom + 128u;
+      const uint32_t d_dom = tmem + kSlabAccCol, d_small = d_dom + 128u;
       int64_t it = 0;
       for (int64_t sl = blockIdx.x; sl < p.nslab && ok; sl += gridDim.x, ++it) {
         const uint32_t ph = (uint32_t)(it & 1);
         // GEMM 1: A = K2 (tensor memory), B = S split; the accumulator is free
         // once the converters drained GEMM 2 of the previous slab
-        if (!mbar_wait(a2empty, ph ^ 1u, abort_flag, p.err)) break;
+        if (!mbar_wait_warp(a2empty, ph ^ 1u, abort_flag, p.err)) break;
         uint32_t acc_small = 0;
         for (int kb = 0; kb < 2 && ok; ++kb) {
-          if (!mbar_wait(&bfull[kb], ph, abort_flag, p.err)) {
+          if (!mbar_wait_warp(&bfull[kb], ph, abort_flag, p.err)) {
             ok = false;
             break;
           }
@@ -1896,25 +1902,25 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 #pragma unroll
               for (int tv = 0; tv < TV; ++tv) {
                 if (ti + tv >= kMaxT) continue;
-                const uint32_t a = tmem_base + (uint32_t)(ti * 64 + kb * 32 + kk * 8);
+                const uint32_t a = tmem + (uint32_t)(ti * 64 + kb * 32 + kk * 8);
                 const uint64_t bd =
                     bdesc0 + (((uint32_t)kb * kKbBytes + (uint32_t)tv * kFsBTermBytes +
                                (uint32_t)kk * 32u) >> 4);
                 if (ti == 0 && tv == 0) {
-                  mma_bf16_ta(d_dom, a, bd, idesc, (kb | kk) ? 1u : 0u);
+                  mma_one_ta(d_dom, a, bd, idesc, (kb | kk) ? 1u : 0u, elect);
                 } else {
-                  mma_bf16_ta(d_small, a, bd, idesc, acc_small);
+                  mma_one_ta(d_small, a, bd, idesc, acc_small, elect);
                   acc_small = 1;
                 }
               }
         }
         if (!ok) break;
-        mma_commit(a1full);
+        mma_commit_one(a1full, elect);
         // GEMM 2: A = K3 (shared memory), B = U split, one k block at a time
-        if (!mbar_wait(a1empty, ph, abort_flag, p.err)) break;
+        if (!mbar_wait_warp(a1empty, ph, abort_flag, p.err)) break;
         acc_small = 0;
         for (int kb = 0; kb < 2 && ok; ++kb) {
-          if (!mbar_wait(&ufull[kb], ph, abort_flag, p.err)) {
+          if (!mbar_wait_warp(&ufull[kb], ph, abort_flag, p.err)) {
             ok = false;
             break;
           }
@@ -1932,19 +1938,19 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
                     bdesc0 + (((uint32_t)kb * kKbBytes + (uint32_t)tv * kFsBTermBytes +
                                (uint32_t)kk * 32u) >> 4);
                 if (ti == 0 && tv == 0) {
-                  mma_bf16(d_dom, ad, bd, idesc, (kb | kk) ? 1u : 0u);
+                  mma_one(d_dom, ad, bd, idesc, (kb | kk) ? 1u : 0u, elect);
                 } else {
-                  mma_bf16(d_small, ad, bd, idesc, acc_small);
+                  mma_one(d_small, ad, bd, idesc, acc_small, elect);
                   acc_small = 1;
                 }
               }
-          mma_commit(&bfree[kb]);
+          mma_commit_one(&bfree[kb], elect);
         }
         if (!ok) break;
-        mma_commit(a2full);
+        mma_commit_one(a2full, elect);
       }
-      mma_commit(drain);
-      mbar_wait_own(drain, 0, p.err);
+      mma_commit_one(drain, elect);
+      if (elect) mbar_wait_own(drain, 0, p.err);
     }
     __syncwarp();
   } else {

@@ -157,7 +157,7 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
 // As mma_bf16 (operand formats are the instruction descriptor's), issued by the one lane whose `elect` is 1 without a branch, for
 // a warp that runs its loop convergently: descriptors then stay in uniform
 // registers (inside a lane == 0 branch every MMA first moves them there).
-__device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+__device__ __forceinline__ void mma_one(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                              uint32_t idesc, uint32_t accumulate,
                                              uint32_t elect) {
   asm volatile(
@@ -169,6 +169,19 @@ __device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint64_t adesc, uin
       : "memory");
 }
 
+// The same with the A operand in tensor memory.
+__device__ __forceinline__ void mma_one_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                           uint32_t idesc, uint32_t accumulate,
+                                           uint32_t elect) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(elect)
+      : "memory");
+}
+
 __device__ __forceinline__ void mma_commit_one(uint64_t* bar, uint32_t elect) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"
@@ -176,6 +189,12 @@ __device__ __forceinline__ void mma_commit_one(uint64_t* bar, uint32_t elect) {
       "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
           smem_u32(bar)), "r"(elect)
       : "memory");
+}
+
+// A bounded wait of a whole converged warp.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
+                                               volatile int* abort_flag, int* err) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err));
 }
 
 // 1 in one lane of a converged warp, 0 in the others.

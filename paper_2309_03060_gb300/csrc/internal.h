@@ -205,10 +205,21 @@ void bilinear(Ctx* c, const cola_linop* op, const T* Uw, const T* X, int64_t R, 
 void collect_leaves(const cola_linop* op, std::vector<const cola_linop*>& out);
 
 // ------------------------------------------------------------- kernels API
+// Diagonal term of a product's epilogue: C += coeff d (.) x, x laid out as C
+// (same strides and batch stride), d[offset within one batch entry] per element
+// (dstride != 0) or d[0].
+template <typename T>
+struct GemmDiag {
+  const T* x = nullptr;
+  const T* d = nullptr;
+  int64_t dstride = 0;
+  double coeff = 0.0;
+};
 template <typename T>
 void gemm(Ctx* c, int64_t M, int64_t N, int64_t K, double alpha, const T* A, int64_t lda_m,
           int64_t lda_k, int64_t sA, const T* B, int64_t ldb_k, int64_t ldb_n, int64_t sB,
-          double beta, T* C, int64_t ldc_m, int64_t ldc_n, int64_t sC, int64_t batch);
+          double beta, T* C, int64_t ldc_m, int64_t ldc_n, int64_t sC, int64_t batch,
+          const GemmDiag<T>& dg = {});
 
 // One problem of a grouped GEMM: C = alpha A B + beta C with element strides.
 template <typename T>
@@ -326,6 +337,10 @@ int* tc_errflag(Ctx* c);            // device flag the tensor-core kernels raise
 bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, const double* X,
                       int64_t size_in, const double* F, int64_t f_i, int64_t f_j, double beta,
                       double* Y, int64_t size_out, int64_t R);
+// Y = (c_k Kron + c_d Diag(d)) X with the diagonal term in the last kernel's
+// epilogue; false (nothing launched) when the Kronecker node has no split form.
+bool kron_tc_shift_apply(Ctx* c, const cola_linop* kron, const cola_linop* dg, const float* X,
+                         float* Y, int64_t R, double ck, double cd, int depth);
 // Fused MIXED CG MVM for Sum(Kron, Diag); see kron_tc.cu.  0 = not applicable.
 // p_new = z + beta p_old is formed in the first mode step (p_new != p_old).
 // rev: the first mode step walks its tiles in reverse order (and the slab

@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <atomic>
 #include <cmath>
 
@@ -271,6 +272,42 @@ template <typename T>
 void kron_tc_apply(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coeff,
                    double beta, int depth, bool tr);  // kron_tc.cu
 
+// The d mode steps of Y = coeff Kron X + beta Y [+ the diagonal term dg] on the SIMT
+// cores or, in FP64, as digit products (gemm's choice).
+template <typename T>
+static void kron_steps(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coeff,
+                       double beta, int depth, bool tr, const GemmDiag<T>& dg) {
+  // Cyclic mode products: step k contracts the leading index of the
+  // current layout [j_k, rest] into [rest, i_k]; after d steps the layout
+  // is back in (i_1, ..., i_d) order.
+  const int d = (int)op->kids.size();
+  int64_t cur_size = tr ? op->rows : op->cols;
+  int64_t maxsz = cur_size;
+  for (int k = 0; k < d; ++k) {
+    const cola_linop* f = op->kids[k];
+    const int64_t n_in = tr ? f->rows : f->cols, n_out = tr ? f->cols : f->rows;
+    cur_size = cur_size / n_in * n_out;
+    maxsz = std::max(maxsz, cur_size);
+  }
+  cur_size = tr ? op->rows : op->cols;
+  const T* cur = X;
+  for (int k = 0; k < d; ++k) {
+    const cola_linop* f = op->kids[k];
+    const T* F = leaf_ptr<T>(f);
+    const int64_t ld = leaf_ld(f);
+    const int64_t n_in = tr ? f->rows : f->cols, n_out = tr ? f->cols : f->rows;
+    const int64_t rest = cur_size / n_in, out_size = rest * n_out;
+    const bool last = (k == d - 1);
+    T* dst = last ? Y : tmp<T>(c, "kron", depth, k & 1, maxsz * R);
+    // B[k=j, n=i] = F_op[i, j]
+    const int64_t lbk = tr ? ld : 1, lbn = tr ? 1 : ld;
+    gemm<T>(c, rest, n_out, n_in, last ? coeff : 1.0, cur, 1, rest, cur_size, F, lbk, lbn, 0,
+            last ? beta : 0.0, dst, n_out, 1, out_size, R, last ? dg : GemmDiag<T>{});
+    cur = dst;
+    cur_size = out_size;
+  }
+}
+
 template <typename T>
 void apply(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coeff, double beta,
            int depth, bool tr, int prec) {
@@ -305,6 +342,23 @@ void apply(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coe
     }
     case LK_SUM: {
       size_t i0 = 0;
+      // a Kronecker product and a diagonal term: one pass over X and Y fewer
+      if (op->kids.size() == 2) {
+        const int ik = op->kids[0]->kind == LK_KRON ? 0 : 1, id = 1 - ik;
+        const cola_linop *kr = op->kids[ik], *dg = op->kids[id];
+        if (kr->kind == LK_KRON && dg->kind == LK_DIAG) {
+          const double ck = coeff * op->coeffs[ik], cd = coeff * op->coeffs[id];
+          if (std::is_same<T, double>::value) {
+            kron_steps<T>(c, kr, X, Y, R, ck, beta, depth + 1, tr,
+                          GemmDiag<T>{X, leaf_ptr<T>(dg), dg->stride, cd});
+            break;
+          }
+          if constexpr (std::is_same<T, float>::value) {
+            if (!tr && beta == 0.0 && kron_tc_shift_apply(c, kr, dg, X, Y, R, ck, cd, depth + 1))
+              break;
+          }
+        }
+      }
       // a tridiagonal Kronecker sum followed by a diagonal term: one pass
       const cola_linop* k0 = op->kids[0];
       if (op->kids.size() >= 2 && k0->kind == LK_KRONSUM && k0->tridiag &&
@@ -344,35 +398,7 @@ void apply(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coe
         kron_tc_apply<T>(c, op, X, Y, R, coeff, beta, depth, tr);
         break;
       }
-      // Cyclic mode products: step k contracts the leading index of the
-      // current layout [j_k, rest] into [rest, i_k]; after d steps the layout
-      // is back in (i_1, ..., i_d) order.
-      const int d = (int)op->kids.size();
-      int64_t cur_size = tr ? op->rows : op->cols;
-      int64_t maxsz = cur_size;
-      for (int k = 0; k < d; ++k) {
-        const cola_linop* f = op->kids[k];
-        const int64_t n_in = tr ? f->rows : f->cols, n_out = tr ? f->cols : f->rows;
-        cur_size = cur_size / n_in * n_out;
-        maxsz = std::max(maxsz, cur_size);
-      }
-      cur_size = tr ? op->rows : op->cols;
-      const T* cur = X;
-      for (int k = 0; k < d; ++k) {
-        const cola_linop* f = op->kids[k];
-        const T* F = leaf_ptr<T>(f);
-        const int64_t ld = leaf_ld(f);
-        const int64_t n_in = tr ? f->rows : f->cols, n_out = tr ? f->cols : f->rows;
-        const int64_t rest = cur_size / n_in, out_size = rest * n_out;
-        const bool last = (k == d - 1);
-        T* dst = last ? Y : tmp<T>(c, "kron", depth, k & 1, maxsz * R);
-        // B[k=j, n=i] = F_op[i, j]
-        const int64_t lbk = tr ? ld : 1, lbn = tr ? 1 : ld;
-        gemm<T>(c, rest, n_out, n_in, last ? coeff : 1.0, cur, 1, rest, cur_size, F, lbk, lbn, 0,
-                last ? beta : 0.0, dst, n_out, 1, out_size, R);
-        cur = dst;
-        cur_size = out_size;
-      }
+      kron_steps<T>(c, op, X, Y, R, coeff, beta, depth, tr, GemmDiag<T>{});
       break;
     }
     case LK_KRONSUM: {

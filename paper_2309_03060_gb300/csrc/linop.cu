@@ -348,7 +348,7 @@ void apply(Ctx* c, const cola_linop* op, const T* X, T* Y, int64_t R, double coe
         const cola_linop *kr = op->kids[ik], *dg = op->kids[id];
         if (kr->kind == LK_KRON && dg->kind == LK_DIAG) {
           const double ck = coeff * op->coeffs[ik], cd = coeff * op->coeffs[id];
-          if (std::is_same<T, double>::value) {
+          if (prec != COLA_PREC_MIXED || std::is_same<T, double>::value) {
             kron_steps<T>(c, kr, X, Y, R, ck, beta, depth + 1, tr,
                           GemmDiag<T>{X, leaf_ptr<T>(dg), dg->stride, cd});
             break;

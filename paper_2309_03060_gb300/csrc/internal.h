@@ -308,6 +308,27 @@ struct CgState {
   int restart;  // set by a residual replacement that restarts the search direction
 };
 
+// CG iteration with U read once (cg_lowrank.cu), for a Sum of a tridiagonal
+// two-factor Kronecker sum, a symmetric low-rank term and at most one diagonal.
+struct LrCg {
+  bool on = false;
+  int n1 = 0, n2 = 0, rank = 0, S = 1, nb_pq = 0, nb_up = 0;
+  int64_t rpb = 0, dstride = 0;
+  float cs = 0.0f, cd = 0.0f;
+  double cu = 0.0;
+  const float *U = nullptr, *bands = nullptr, *d = nullptr;
+  float *q = nullptr, *p2 = nullptr, *w32 = nullptr;
+  double *part = nullptr, *part_rz = nullptr, *part_rr = nullptr, *part_w = nullptr;
+  double *W = nullptr, *Wz = nullptr, *vtx = nullptr;
+};
+// Fills L (leaves prepared in FP32, workspace sized); false when op has another form.
+bool lr_cg_setup(Ctx* c, const cola_linop* op, int64_t R, LrCg* L);
+void lr_cg_refresh(Ctx* c, const LrCg& L, const float* z, int64_t R);
+// One iteration up to the new r, x and the partials of r . z, r . r (part_rz,
+// part_rr, nb_up per right-hand side); the caller runs the beta kernel.
+void lr_cg_step(Ctx* c, const LrCg& L, const float* p_old, float* p_new, float* r, float* x,
+                const float* invd, CgState* st, int64_t R);
+
 // ------------------------------------------------------------ solver entries
 cola_status cg_solve_impl(Ctx* c, const cola_linop* op, const void* B, void* X, int64_t R,
                           const cola_cg_opts& o, cola_cg_info* info);

@@ -909,6 +909,7 @@ struct CgBufs {
   bool defer_x;           // x updated every kPRing iterations from the ring (fused FP32)
   double* alpha_hist;     // [kPRing][R] alpha of each ring slot
   T* invd;
+  LrCg lr;                // stencil + diagonal + low rank: U read once per iteration
   KronPrecond kp;         // kron_precond: z = M^-1 r by the eigen-structured solve
   bool kprec;
   double *x64, *b64, *r64;
@@ -981,9 +982,30 @@ static void precond_z(Ctx* c, CgBufs<T>& B, int64_t N, int64_t R, int nblk) {
   c->count_launch();
 }
 
+// U^T z of a z formed outside the iteration (start, replacement, verification).
+template <typename T>
+static void lr_refresh(Ctx* c, CgBufs<T>& B, int64_t R) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (B.lr.on) lr_cg_refresh(c, B.lr, z_of(B), R);
+  }
+}
+
 template <typename T>
 static void cg_iteration(Ctx* c, const cola_linop* op, CgBufs<T>& B, int64_t N, int64_t R,
                          int nblk, int prec, double delta2, int refine, bool defer) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (B.lr.on) {
+      const int nxt = B.cur ^ 1;
+      lr_cg_step(c, B.lr, B.pp[B.cur], B.pp[nxt], B.r, B.x, B.invd, B.st, R);
+      B.cur = nxt;
+      B.p = B.pp[nxt];
+      k_cg_beta<<<(unsigned)R, 256, 0, c->s>>>(B.st, B.lr.part_rz, B.lr.part_rr, B.lr.nb_up,
+                                                delta2, refine, B.beta_vec);
+      c->count_launch();
+      COLA_CUDA(cudaGetLastError());
+      return;
+    }
+  }
   if (B.fused_tiles > 0) {
     // p_new = z + beta p_old (first mode step), Ap and p^T A p partials (last)
     const int nxt = (B.cur + 1) % kPRing;
@@ -1170,6 +1192,10 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                  "kron_precond takes c_k Kron(K_1..K_d) + c_d Diag(d) with square dense factors");
   }
 
+  if constexpr (std::is_same<T, float>::value) {
+    if (!B.kprec && B.ro_cap == 0 && lr_cg_setup(c, op, R, &B.lr)) B.pp[1] = B.lr.p2;
+  }
+
   if (refine) {
     B.x64 = (double*)ws.get("cg.x64", 8 * N * R);
     B.b64 = (double*)ws.get("cg.b64", 8 * N * R);
@@ -1198,6 +1224,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                                                          B.z, nblk, B.part_rz, B.part_rr);
   c->count_launch();
   precond_z<T>(c, B, N, R, nblk);
+  lr_refresh<T>(c, B, R);
   k_cg_restate<<<(unsigned)((R + 127) / 128), 128, 0, c->s>>>(
       B.st, B.part_rz, B.part_rr, nblk, R, refine ? rr64 : nullptr, bb, o.tol, 1, nullptr);
   c->count_launch();
@@ -1221,6 +1248,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
   // chunks keep the replacements (and restarts) close behind it
   if (B.kprec) chunk = std::min(chunk, kPRing);
   if (B.fused_tiles > 0) chunk = (chunk + kPRing - 1) / kPRing * kPRing;
+  if (B.lr.on) chunk = (chunk + 1) / 2 * 2;  // two p buffers
   // Without refinement the iterations after the last right-hand side stopped are
   // lost, and nothing else depends on where a chunk ends: chunks start at 8
   // iterations and grow (up to `chunk`) until one takes kChunkSeconds, well above
@@ -1320,6 +1348,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                                                              B.part_rz, B.part_rr);
       c->count_launch();
       precond_z<T>(c, B, N, R, nblk);
+      lr_refresh<T>(c, B, R);
       k_cg_restate<<<(unsigned)((R + 127) / 128), 128, 0, c->s>>>(
           B.st, B.part_rz, B.part_rr, nblk, R, rr64, bb, o.tol, 0, B.beta_vec);
       c->count_launch();
@@ -1348,6 +1377,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                                                            B.part_rz, B.part_rr);
     c->count_launch();
     precond_z<T>(c, B, N, R, nblk);
+    lr_refresh<T>(c, B, R);
     k_cg_verify<<<(unsigned)((R + 127) / 128), 128, 0, c->s>>>(B.st, B.part_rz, B.part_rr, nblk,
                                                                R, B.beta_vec);
     c->count_launch();

@@ -329,6 +329,27 @@ void lr_cg_refresh(Ctx* c, const LrCg& L, const float* z, int64_t R);
 void lr_cg_step(Ctx* c, const LrCg& L, const float* p_old, float* p_new, float* r, float* x,
                 const float* invd, CgState* st, int64_t R);
 
+// CG loop of small Kronecker operators in one cooperative kernel (cg_small.cu).
+struct SmallCg {
+  bool on = false;
+  const cola_linop *kron = nullptr, *diag = nullptr;
+  double ck = 1.0, cd = 0.0;
+  int tiles2 = 0, tiles = 0;
+  void *t = nullptr, *p1 = nullptr;
+  double* part = nullptr;
+  int* act = nullptr;
+  unsigned* bar = nullptr;
+};
+// Fills S for Kron(K_1, K_2) [+ Diag] of at most 608 4 x 8 output tiles over all
+// right-hand sides; false for another operator.
+template <typename T>
+bool small_cg_setup(Ctx* c, const cola_linop* op, int64_t R, SmallCg* S);
+// Up to `limit` iterations from the state in st, r, x and the direction p (the
+// same meaning as between two iterations of the general path, unrefined).
+template <typename T>
+void small_cg_run(Ctx* c, const SmallCg& S, T* r, T* x, T* p, const T* invd, CgState* st,
+                  int64_t R, int limit);
+
 // ------------------------------------------------------------ solver entries
 cola_status cg_solve_impl(Ctx* c, const cola_linop* op, const void* B, void* X, int64_t R,
                           const cola_cg_opts& o, cola_cg_info* info);

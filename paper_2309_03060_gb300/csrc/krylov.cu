@@ -73,6 +73,8 @@ constexpr double kDeferRatio = 100.0;
 constexpr double kRestartGap2 = 100.0;
 // Host time a graph chunk of an unrefined solve grows to (see cg_run).
 constexpr double kChunkSeconds = 400e-6;
+// Iterations per launch of the one-kernel CG loop (bounds a launch to ~30 ms).
+constexpr int kSmallChunk = 2048;
 
 // alpha = r^T z / p^T A p, with p^T A p the ordered sum of nparts partials.
 // One block per right-hand side: p^T A p from its partial sums, alpha = r^T z / p^T A p.
@@ -909,6 +911,7 @@ struct CgBufs {
   bool defer_x;           // x updated every kPRing iterations from the ring (fused FP32)
   double* alpha_hist;     // [kPRing][R] alpha of each ring slot
   T* invd;
+  SmallCg small;          // the whole loop in one kernel (small Kronecker operators)
   LrCg lr;                // stencil + diagonal + low rank: U read once per iteration
   KronPrecond kp;         // kron_precond: z = M^-1 r by the eigen-structured solve
   bool kprec;
@@ -1192,6 +1195,8 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                  "kron_precond takes c_k Kron(K_1..K_d) + c_d Diag(d) with square dense factors");
   }
 
+  if (!refine && prec != COLA_PREC_MIXED && !B.kprec && B.ro_cap == 0)
+    small_cg_setup<T>(c, op, R, &B.small);
   if constexpr (std::is_same<T, float>::value) {
     if (!B.kprec && B.ro_cap == 0 && lr_cg_setup(c, op, R, &B.lr)) B.pp[1] = B.lr.p2;
   }
@@ -1295,13 +1300,29 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
   bool any_active = false;
   for (int64_t r = 0; r < R; ++r) any_active |= hst[r].active != 0;
   // one eager iteration sizes every workspace buffer before capture
-  if (any_active && o.maxiter > 0) {
+  if (any_active && o.maxiter > 0 && !B.small.on) {
     cg_iteration<T>(c, op, B, N, R, nblk, prec, delta2, refine ? 1 : 0, false);
     iters = 1;
   }
   for (int verify = 0;; ++verify) {
   while (any_active) {
     if (iters >= cap) break;
+    if (B.small.on) {
+      // ends by itself when every right-hand side has stopped
+      small_cg_run<T>(c, B.small, B.r, B.x, B.p, B.invd, B.st, R,
+                      (int)std::min<int64_t>(cap - iters, kSmallChunk));
+      read_state();
+      any_active = false;
+      int64_t most = 0;
+      for (int64_t r = 0; r < R; ++r) {
+        any_active |= hst[r].active != 0;
+        most = std::max<int64_t>(most, hst[r].iters);
+      }
+      if (most <= iters) tc_check_error(c);  // no progress: the kernel gave up
+      iters = std::max(most, iters + (most <= iters ? 1 : 0));
+      trace_line("chunk");
+      continue;
+    }
     const auto tc0 = std::chrono::steady_clock::now();
     cg_chunk<T>(c, op, B, N, R, nblk, prec, delta2, refine ? 1 : 0, run_chunk, graph_key());
     iters += run_chunk;

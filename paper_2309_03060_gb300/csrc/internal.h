@@ -390,6 +390,8 @@ bool kron_tc_shift_apply(Ctx* c, const cola_linop* kron, const cola_linop* dg, c
 int64_t kron_tc_cg_mvm(Ctx* c, const cola_linop* op, const float* z, const double* beta_vec,
                        const float* p_old, float* p_new, float* Ap, double* tile_dot, int64_t R,
                        int depth, int rev = 0);
+// Most tiles per right-hand side that kron_tc_cg_mvm and kron_tc_lanczos_mvm use
+// (they return the number; 8 partials per tile).
 int64_t kron_tc_tiles_per_rhs(const cola_linop* op);
 // Fused Lanczos MIXED MVM for Sum(Kron, scalar Diag); see kron_tc.cu.  0 = not applicable.
 int64_t kron_tc_lanczos_mvm(Ctx* c, const cola_linop* op, const float* w_in,

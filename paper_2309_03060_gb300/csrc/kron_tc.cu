@@ -1206,12 +1206,16 @@ __global__ void __launch_bounds__(kPresplitThreads) k_presplit_tab(const TcGemmP
   }
 }
 
-template <int TF, int TV, class Src>
+// NT: rows (right-hand-side entries) per tile; a product with too few 128-row
+// tiles to reach every SM takes 64 or 32 (gemm_row_tile).
+template <int TF, int TV, class Src, int NT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     k_kron_tc_gemm(const __grid_constant__ Src src, const TcGemmLaunch L) {
   constexpr int kMaxT = TF > TV ? TF : TV;
   constexpr bool kSmall = TF > 1 || TV > 1;
-  constexpr uint32_t kStageBytes = (uint32_t)(TF + TV) * kGemmTermBytes;
+  constexpr uint32_t kXBytes = (uint32_t)NT * 128u;  // one X term: NT rows x 64 BF16
+  constexpr uint32_t kStageBytes = (uint32_t)TV * kXBytes + (uint32_t)TF * kGemmTermBytes;
+  constexpr int NC = NT / 2;  // rows an epilogue warp drains
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* full = (uint64_t*)(base + (size_t)L.stages * kStageBytes);  // [stages]
@@ -1265,7 +1269,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const TcGemmParams& p = src.get(t, lt);
         const int nc = (int)(lt % p.nchunks);
         const int64_t tm = lt / p.nchunks;
-        const int64_t r = tm / p.tiles_m, m0 = (tm % p.tiles_m) * kTileM;
+        const int64_t r = tm / p.tiles_m, m0 = (tm % p.tiles_m) * NT;
         // the tile's fields in registers (a problem table in global memory
         // would be re-read after every asm statement of the loop below)
         const int kblocks = p.kblocks, img_rows = p.img_rows;
@@ -1285,17 +1289,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 #pragma unroll
           for (int tv = 0; tv < TV; ++tv) {
             if constexpr (Src::kTma)
-              tma_load_2d(st + tv * kGemmTermBytes, &p.tm_x, kb * kBlockK,
+              tma_load_2d(st + tv * kXBytes, &p.tm_x, kb * kBlockK,
                           (int)(tv * xrows) + y0, &full[s]);
             else
-              bulk_g2s(st + tv * kGemmTermBytes,
+              bulk_g2s(st + tv * kXBytes,
                        ximg + (((size_t)tv * kblocks + kb) * (size_t)rows_pad + (size_t)xrow0) *
                                   kBlockK,
-                       kGemmTermBytes, &full[s]);
+                       kXBytes, &full[s]);
           }
 #pragma unroll
           for (int ti = 0; ti < TF; ++ti)
-            bulk_g2s(st + (TV + ti) * kGemmTermBytes,
+            bulk_g2s(st + TV * kXBytes + ti * kGemmTermBytes,
                      bimg + (((size_t)ti * kblocks + kb) * (size_t)img_rows +
                                (size_t)nc * kTileM) * kBlockK,
                      kGemmTermBytes, &full[s]);
@@ -1318,7 +1322,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     {
       const uint32_t elect = elect_one();
       const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);  // warp-uniform
-      constexpr uint32_t idesc = idesc_bf16(kTileM, kTileM);  // M = outputs, N = rows
+      constexpr uint32_t idesc = idesc_bf16(kTileM, NT);  // M = outputs, N = rows
       bool ok = true;
       if (L.stall_ns)
         ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, L.err, L.stall_ns));
@@ -1350,9 +1354,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
               for (int tv = 0; tv < TV; ++tv) {
                 if (ti + tv >= kMaxT) continue;
                 const uint64_t ad =
-                    sw128_desc(st + (uint32_t)(TV + ti) * kGemmTermBytes + (uint32_t)kk * 32u);
+                    sw128_desc(st + (uint32_t)TV * kXBytes + (uint32_t)ti * kGemmTermBytes +
+                               (uint32_t)kk * 32u);
                 const uint64_t bd =
-                    sw128_desc(st + (uint32_t)tv * kGemmTermBytes + (uint32_t)kk * 32u);
+                    sw128_desc(st + (uint32_t)tv * kXBytes + (uint32_t)kk * 32u);
                 if (ti == 0 && tv == 0) {
                   mma_one(d_big, ad, bd, idesc, acc_big, elect);
                   acc_big = 1;
@@ -1394,11 +1399,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const float d0 = (p.epi_x && p.epi_dstride == 0) ? p.epi_d[0] : 0.0f;
       const int nc = (int)(lt % p.nchunks);
       const int64_t tm = lt / p.nchunks;
-      const int64_t r = tm / p.tiles_m, m0 = (tm % p.tiles_m) * kTileM;
-      const uint32_t taddr = tmem_base + lane_off + (uint32_t)b * 256u + (uint32_t)chalf * 64u;
+      const int64_t r = tm / p.tiles_m, m0 = (tm % p.tiles_m) * NT;
+      const uint32_t taddr = tmem_base + lane_off + (uint32_t)b * 256u + (uint32_t)chalf * (uint32_t)NC;
       const int i = nc * kTileM + il;
-      const int64_t mbase = m0 + chalf * 64;
-      const int nrows = (int)((p.rest - mbase < 64) ? (p.rest - mbase) : 64);
+      const int64_t mbase = m0 + chalf * NC;
+      const int nrows = (int)((p.rest - mbase < NC) ? (p.rest - mbase) : NC);  // may be < 0
       const bool live = i < p.n_out && nrows > 0;
       const int64_t ld = p.n_out;
       float* yp = p.Y + r * p.size_out + mbase * ld + i;
@@ -1414,12 +1419,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       uint16_t* const oimg = p.oimg;
       const int64_t o_rstride = p.o_rstride, o_rows = p.o_rows;
       const int o_kpad = p.o_kpad, o_swz = p.o_swz;
-      float part = 0.0f;  // this thread's <= 64 products of x . y
+      float part = 0.0f;  // this thread's <= NC products of x . y
       if (!ex && beta == 0.0f) {
         // plain step: the whole accumulator into registers, released, stored
-        float a[64];
+        float a[NC];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < NC / 8; ++q) {
           uint32_t v[8], w[8];
           tmem_ld8(taddr + (uint32_t)(q * 8), v);
           if (kSmall) tmem_ld8(taddr + 128u + (uint32_t)(q * 8), w);
@@ -1431,13 +1436,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
         tc_fence_before();
         mbar_arrive(&aempty[b]);
-        if (live && oimg) {
-          // row i (this step's output) of the next step's image, its 64 k
-          // (this step's rows mbase ..) in TV split terms, zero past rest
+        // (128-row tiles: a half with no rows has no image columns either)
+        const bool put = NT == kTileM ? live : i < (int)ld && mbase < o_kpad;
+        if (put && oimg) {
+          // row i (this step's output) of the next step's image, its k (this
+          // step's rows mbase ..) in TV split terms, zero past rest up to o_kpad
           const int64_t row = r * o_rstride + i;
           const int kb = (int)(mbase / kBlockK);
+          const int ch0 = NT == kTileM ? 0 : (int)(mbase % kBlockK) / 8;
 #pragma unroll
-          for (int ch = 0; ch < 8; ++ch) {
+          for (int ch = 0; ch < NC / 8; ++ch) {
             uint32_t w[3][4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -1452,27 +1460,27 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int tv = 0; tv < TV; ++tv) {
               const size_t pos =
                   o_swz ? (((size_t)tv * (o_kpad / kBlockK) + kb) * (size_t)o_rows + row) * kBlockK +
-                              (size_t)((ch ^ (int)(row & 7)) * 8)
+                              (size_t)(((ch0 + ch) ^ (int)(row & 7)) * 8)
                         : ((size_t)tv * o_rows + row) * o_kpad + mbase + ch * 8;
               *reinterpret_cast<uint4*>(oimg + pos) = make_uint4(w[tv][0], w[tv][1], w[tv][2], w[tv][3]);
             }
           }
-        } else if (live) {
+        } else if (live && !oimg) {
 #pragma unroll
-          for (int c = 0; c < 64; ++c)
+          for (int c = 0; c < NC; ++c)
             if (c < nrows) yp[c * ld] = a[c];
         }
         continue;
       }
       if (ex && !ed && !eq && beta == 0.0f) {
-        // the CG step: x for all 64 rows first (one global latency; loads
+        // the CG step: x for all rows first (one global latency; loads
         // issued after a store to a buffer the compiler cannot prove distinct
         // would wait for it), then 16 rows at a time from the accumulator
-        float xa[64];
+        float xa[NC];
 #pragma unroll
-        for (int c = 0; c < 64; ++c) xa[c] = (live && c < nrows) ? __ldg(ex + c * ld) : 0.0f;
+        for (int c = 0; c < NC; ++c) xa[c] = (live && c < nrows) ? __ldg(ex + c * ld) : 0.0f;
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
+        for (int h = 0; h < NC / 16; ++h) {
           uint32_t v[16], w[16];
           tmem_ld8(taddr + (uint32_t)(h * 16), v);
           tmem_ld8(taddr + (uint32_t)(h * 16 + 8), v + 8);
@@ -1496,7 +1504,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         // 16 rows at a time: accumulator columns, every load of the group, then
         // its stores (loads interleaved with the stores would wait for them)
 #pragma unroll 1
-        for (int h = 0; h < 4; ++h) {
+        for (int h = 0; h < NC / 16; ++h) {
           uint32_t v[16], w[16];
           tmem_ld8(taddr + (uint32_t)(h * 16), v);
           tmem_ld8(taddr + (uint32_t)(h * 16 + 8), v + 8);
@@ -2326,15 +2334,16 @@ static bool fs_plan(const TcParams& p, TcFsParams& r) {
   return true;
 }
 
-// BF16 image [rows][cols] of the GEMM path's X image, box 64 columns x 128
+// BF16 image [rows][cols] of the GEMM path's X image, box 64 columns x box_rows
 // rows, 128-byte swizzle (the UMMA K-major layout); reads past the rows
 // return zeros.
-static bool tmap_image(CUtensorMap* m, const uint16_t* base, int64_t rows, int64_t cols) {
+static bool tmap_image(CUtensorMap* m, const uint16_t* base, int64_t rows, int64_t cols,
+                       int box_rows) {
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)kTileM};
+  const cuuint32_t box[2] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(base), dims, strides,
              box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -2343,13 +2352,36 @@ static bool tmap_image(CUtensorMap* m, const uint16_t* base, int64_t rows, int64
 
 template <class Src>
 using GemmKernel = void (*)(Src, TcGemmLaunch);
-template <class Src>
-static GemmKernel<Src> gemm_kernel(int tf, int tv) {
+template <class Src, int NT>
+static GemmKernel<Src> gemm_kernel_nt(int tf, int tv) {
   static const GemmKernel<Src> tab[3][3] = {
-      {k_kron_tc_gemm<1, 1, Src>, k_kron_tc_gemm<1, 2, Src>, k_kron_tc_gemm<1, 3, Src>},
-      {k_kron_tc_gemm<2, 1, Src>, k_kron_tc_gemm<2, 2, Src>, k_kron_tc_gemm<2, 3, Src>},
-      {k_kron_tc_gemm<3, 1, Src>, k_kron_tc_gemm<3, 2, Src>, k_kron_tc_gemm<3, 3, Src>}};
+      {k_kron_tc_gemm<1, 1, Src, NT>, k_kron_tc_gemm<1, 2, Src, NT>,
+       k_kron_tc_gemm<1, 3, Src, NT>},
+      {k_kron_tc_gemm<2, 1, Src, NT>, k_kron_tc_gemm<2, 2, Src, NT>,
+       k_kron_tc_gemm<2, 3, Src, NT>},
+      {k_kron_tc_gemm<3, 1, Src, NT>, k_kron_tc_gemm<3, 2, Src, NT>,
+       k_kron_tc_gemm<3, 3, Src, NT>}};
   return tab[tf - 1][tv - 1];
+}
+template <class Src>
+static GemmKernel<Src> gemm_kernel(int tf, int tv, int nt) {
+  if constexpr (Src::kTma) {
+    if (nt == 32) return gemm_kernel_nt<Src, 32>(tf, tv);
+    if (nt == 64) return gemm_kernel_nt<Src, 64>(tf, tv);
+  }
+  return gemm_kernel_nt<Src, kTileM>(tf, tv);
+}
+
+// Rows per tile of one split GEMM step: the widest of 128, 64, 32 whose tiles still
+// number at least 3 / 4 of the SMs, 32 when none does.  A tile's factor loads and
+// fixed cost do not shrink with its rows, so wide tiles win once the SMs are
+// busy; below that the step's time is one tile's.  Measured (two 256 x 256 factors, 4
+// right-hand sides, CG iteration): 9.7 us a step with 32 rows (64 tiles), 18.5 us
+// with 128 (16 tiles).
+static int gemm_row_tile(int64_t rest, int64_t R, int nch, int num_sms) {
+  for (int nt = kTileM; nt > 32; nt /= 2)
+    if ((rest + nt - 1) / nt * R * nch * 4 >= (int64_t)num_sms * 3) return nt;
+  return 32;
 }
 using PresplitKernel = void (*)(const float*, int, int64_t, int, int64_t, int, const float*,
                                 const double*, float*, uint16_t*);
@@ -2358,8 +2390,16 @@ static PresplitKernel presplit_kernel(int tv) {
   return tab[tv - 1];
 }
 constexpr int kGemmStages = 2;
-static size_t gemm_smem(int tf, int tv) {
-  return 1024 + (size_t)kGemmStages * (tf + tv) * kGemmTermBytes + 256;
+static size_t gemm_stage(int tf, int tv, int nt) {
+  return (size_t)tv * nt * 128 + (size_t)tf * kGemmTermBytes;
+}
+// Two stages of the widest tile, more of the narrower ones in the same space.
+static int gemm_stages(int tf, int tv, int nt) {
+  return nt == kTileM ? kGemmStages
+                      : (int)std::min<size_t>(4, 200 * 1024 / gemm_stage(tf, tv, nt));
+}
+static size_t gemm_smem(int tf, int tv, int nt) {
+  return 1024 + (size_t)gemm_stages(tf, tv, nt) * gemm_stage(tf, tv, nt) + 256;
 }
 
 // The split GEMM mode step (factor sides above 128): pre-split pass, then the
@@ -2427,8 +2467,9 @@ static uint16_t* gemm_ximage(Ctx* c, const TcParams& p, int depth, int k) {
 // One split GEMM mode step.  `next` (a two-factor product's first step): the
 // epilogue writes the second step's X image instead of Y.  `have_img`: this
 // step's X image was written by the previous step's epilogue (no pre-split).
+// *tiles: tiles per right-hand side.
 static bool gemm_launch(Ctx* c, const cola_linop* f, bool tr, const TcParams& p, int depth,
-                        int k, const TcParams* next = nullptr, bool have_img = false) {
+                        int k, const TcParams* next, bool have_img, int64_t* tiles) {
   if (!gemm_ok(c, p, f, tr)) return false;
   const int kblocks = (p.n_in + kBlockK - 1) / kBlockK, kpad = kblocks * kBlockK;
   const int nch = (p.n_out + kTileM - 1) / kTileM, img_rows = nch * kTileM;
@@ -2436,7 +2477,8 @@ static bool gemm_launch(Ctx* c, const cola_linop* f, bool tr, const TcParams& p,
   const uint16_t* fimg = gemm_factor_image(c, f, tr, p.tf);
   uint16_t* ximg = gemm_ximage(c, p, depth, k);
   TcGemmParams g{};
-  if (!tmap_image(&g.tm_x, ximg, (int64_t)p.tv * xrows, kpad)) return false;
+  const int nt = gemm_row_tile(p.rest, p.batch, nch, c->num_sms);
+  if (!tmap_image(&g.tm_x, ximg, (int64_t)p.tv * xrows, kpad, nt)) return false;
   if (!have_img) {
     const int mode = p.pro_z ? 2 : (p.pro_out ? 1 : 0);
     const dim3 pgrid((unsigned)((p.rest + 63) / 64), (unsigned)(kpad / 64), (unsigned)p.batch);
@@ -2456,9 +2498,11 @@ static bool gemm_launch(Ctx* c, const cola_linop* f, bool tr, const TcParams& p,
   g.Y = p.Y;
   g.rest = p.rest;
   g.size_out = p.size_out;
-  g.tiles_m = p.tiles_m;
+  // a chained first step also writes the zero columns of the image up to o_kpad
+  g.tiles_m = ((next ? (int64_t)g.o_kpad : p.rest) + nt - 1) / nt;
   g.nchunks = nch;
-  g.ntiles = p.tiles_m * p.batch * nch;
+  g.ntiles = g.tiles_m * p.batch * nch;
+  *tiles = g.tiles_m * nch;
   g.xrows = xrows;
   g.n_out = p.n_out;
   g.kblocks = kblocks;
@@ -2472,10 +2516,10 @@ static bool gemm_launch(Ctx* c, const cola_linop* f, bool tr, const TcParams& p,
   g.epi_dot = p.epi_dot;
   g.epi_q2 = p.epi_q2;
   g.epi_gamma = p.epi_gamma;
-  TcGemmLaunch L{kGemmStages, p.err, p.stall_ns};
+  TcGemmLaunch L{gemm_stages(p.tf, p.tv, nt), p.err, p.stall_ns};
   const int grid = (int)std::min<int64_t>(g.ntiles, c->num_sms);
-  launch_pdl(gemm_kernel<GemmOne>(p.tf, p.tv), dim3(grid), dim3(kGemmThreads),
-             gemm_smem(p.tf, p.tv), c->s, GemmOne{g}, L);
+  launch_pdl(gemm_kernel<GemmOne>(p.tf, p.tv, nt), dim3(grid), dim3(kGemmThreads),
+             gemm_smem(p.tf, p.tv, nt), c->s, GemmOne{g}, L);
   c->count_launch();
   COLA_CUDA(cudaGetLastError());
   return true;
@@ -2640,12 +2684,13 @@ static int64_t kron_tc_run(Ctx* c, const cola_linop* op, const float* X, float* 
             COLA_CUDA(cudaFuncSetAttribute(slab_kernel(a, b, em),
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)slab_smem(a, b)));
-          COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmOne>(a, b),
+          for (int nt : {32, 64, kTileM})
+            COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmOne>(a, b, nt),
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)gemm_smem(a, b, nt)));
+          COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmTab>(a, b, kTileM),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gemm_smem(a, b)));
-          COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmTab>(a, b),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)gemm_smem(a, b)));
+                                         (int)gemm_smem(a, b, kTileM)));
         }
       attr_set[c->device] = true;
     }
@@ -2655,8 +2700,10 @@ static int64_t kron_tc_run(Ctx* c, const cola_linop* op, const float* X, float* 
       launch_pdl(fs_kernel(tf, tv), dim3(grid), dim3(kThreadsFs), fs_smem(rp, tv), c->s, rp);
       c->count_launch();
       COLA_CUDA(cudaGetLastError());
-    } else if (!gemm_launch(c, f, tr, p, depth, k, chain && k == 0 ? &p1 : nullptr,
-                            chain && k == 1)) {
+    } else if (int64_t gt = 0; gemm_launch(c, f, tr, p, depth, k, chain && k == 0 ? &p1 : nullptr,
+                                           chain && k == 1, &gt)) {
+      if (last && nsteps == d) last_tiles = gt;
+    } else {
       COLA_REQUIRE(!chain, COLA_ERR_CUDA, "internal: chained split GEMM step not launched");
       COLA_REQUIRE(!p.out_trans, COLA_ERR_UNSUPPORTED,
                    "internal: slab-major output needs the factor-stationary kernel");
@@ -2917,14 +2964,16 @@ int64_t kron_tc_lanczos_slab(Ctx* c, const cola_linop* op, const float* v, const
 }
 
 int64_t kron_tc_tiles_per_rhs(const cola_linop* op) {
-  // row tiles of the last mode step when the operator is Sum(Kron, Diag)
+  // row tiles of the last mode step when the operator is Sum(Kron, Diag), at
+  // most (the split GEMM of sides above 128 may take tiles of 32 rows)
   if (op->kind != LK_SUM || op->kids.size() != 2) return 0;
   for (auto* k : op->kids)
     if (k->kind == LK_KRON && k->kids.size() >= 2 && tc_supported(k)) {
       const cola_linop* last = k->kids.back();
       const int64_t rest = k->rows / last->rows;  // rows produced by the earlier steps
       const int n16 = (int)((last->rows + 15) / 16 * 16);
-      return (rest + kTileM - 1) / kTileM * ((n16 + kChunkMax - 1) / kChunkMax);
+      const int rows = (last->rows > kTileM || last->cols > kTileM) ? 32 : kTileM;
+      return (rest + rows - 1) / rows * ((n16 + kChunkMax - 1) / kChunkMax);
     }
   return 0;
 }
@@ -3191,11 +3240,11 @@ void kron_tc_gemm_batch_launch(Ctx* c, const char* tag, int tf, int tv, bool pre
   L.rev = presplit ? 1 : 0;
   GemmTab src{probs, (const int*)c->ws.bufs.at(tagged(tag, "gtile")).p,
               (const int64_t*)c->ws.bufs.at(tagged(tag, "gfirst")).p, cnt};
-  COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmTab>(tf, tv),
+  COLA_CUDA(cudaFuncSetAttribute(gemm_kernel<GemmTab>(tf, tv, kTileM),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)gemm_smem(tf, tv)));
-  launch_pdl(gemm_kernel<GemmTab>(tf, tv), dim3(c->num_sms), dim3(kGemmThreads),
-             gemm_smem(tf, tv), c->s, src, L);
+                                 (int)gemm_smem(tf, tv, kTileM)));
+  launch_pdl(gemm_kernel<GemmTab>(tf, tv, kTileM), dim3(c->num_sms), dim3(kGemmThreads),
+             gemm_smem(tf, tv, kTileM), c->s, src, L);
   c->count_launch();
   COLA_CUDA(cudaGetLastError());
 }

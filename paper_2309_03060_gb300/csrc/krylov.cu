@@ -1017,13 +1017,16 @@ static void cg_iteration(Ctx* c, const cola_linop* op, CgBufs<T>& B, int64_t N, 
     // odd ring positions: the first mode step runs its tiles backwards, the
     // slab kernel forwards, the residual update backwards; even ones the
     // other way round (each kernel starts where the one before it ended)
-    kron_tc_cg_mvm(c, op, (const float*)z_of(B), B.beta_vec, (const float*)p_old,
-                   (float*)p_new, (float*)B.Ap, B.tile_dot, R, 1, B.cur & 1);
+    const int64_t tiles =
+        kron_tc_cg_mvm(c, op, (const float*)z_of(B), B.beta_vec, (const float*)p_old,
+                       (float*)p_new, (float*)B.Ap, B.tile_dot, R, 1, B.cur & 1);
+    COLA_REQUIRE(tiles > 0 && tiles <= B.fused_tiles, COLA_ERR_UNSUPPORTED,
+                 "internal: fused CG tile count");
     B.cur = nxt;
     B.p = p_new;
     // the small CG kernels launch normally (an early launch measured slower);
     // their pdl_trigger lets the next tensor-core step start its set-up early
-    k_cg_alpha<<<(unsigned)R, 256, 0, c->s>>>(B.st, B.tile_dot, (int)(8 * B.fused_tiles),
+    k_cg_alpha<<<(unsigned)R, 256, 0, c->s>>>(B.st, B.tile_dot, (int)(8 * tiles),
                                                defer ? B.alpha_hist + (int64_t)nxt * R : nullptr);
     c->count_launch();
   } else {
@@ -1743,8 +1746,9 @@ static bool lanczos_fused(Ctx* c, cola_linop* op, const float* Q0, int64_t nv, i
     const float* qprev = q[(j + 1) & 1];
     const int64_t t = kron_tc_lanczos_mvm(c, op, j == 0 ? Q0 : w, scale, qj, qprev, b_cur, w,
                                           tdot, nv, 1);
-    COLA_REQUIRE(t == tiles, COLA_ERR_UNSUPPORTED, "internal: fused Lanczos tile count");
-    k_lz_alpha<<<(unsigned)nv, 256, 0, c->s>>>(st, tdot, (int)(8 * tiles), nv, j, m, alpha,
+    COLA_REQUIRE(t > 0 && t <= tiles, COLA_ERR_UNSUPPORTED,
+                 "internal: fused Lanczos tile count");
+    k_lz_alpha<<<(unsigned)nv, 256, 0, c->s>>>(st, tdot, (int)(8 * t), nv, j, m, alpha,
                                                a_cur);
     c->count_launch();
     k_lz_b<float><<<rows_grid(N, nv, nblk), 256, 0, c->s>>>(N, w, qj, a_cur, nblk, part);

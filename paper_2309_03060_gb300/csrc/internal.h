@@ -383,6 +383,8 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
 // epilogue; false (nothing launched) when the Kronecker node has no split form.
 bool kron_tc_shift_apply(Ctx* c, const cola_linop* kron, const cola_linop* dg, const float* X,
                          float* Y, int64_t R, double ck, double cd, int depth);
+bool kron_tc_scaled_apply(Ctx* c, const cola_linop* kron, const float* s, const float* X,
+                          float* Y, int64_t R, int depth);
 // Fused MIXED CG MVM for Sum(Kron, Diag); see kron_tc.cu.  0 = not applicable.
 // p_new = z + beta p_old is formed in the first mode step (p_new != p_old).
 // rev: the first mode step walks its tiles in reverse order (and the slab

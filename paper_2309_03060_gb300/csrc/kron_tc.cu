@@ -1597,7 +1597,9 @@ struct TcSlabParams {
   const double* gamma;
   const double* scale;   // optional per right-hand side: Y = scale[r] (c_k K x + c_d d[0] x)
                          // - gamma q2, partials of scale[r] x . Y (x unnormalised)
-  const float* d;        // shift scalar (device), term c_d d[0] x
+  const float* d;        // shift scalar (device), term c_d d[0] x; per-element
+                         // variant (EM 3): d of one right-hand side, term c_d d (.) x, or
+                         // Y = c_k d (.) (K S) when x is nullptr
   float coeff, dcoeff;
   int64_t nslab, slabs_per_rhs;
   double* dot;           // [nslab][8] partials of x . Y
@@ -1720,11 +1722,12 @@ __device__ __forceinline__ void slab_drain16(uint32_t taddr, float* a) {
 }
 
 // EM: 0 Y = c_k K S; 1 adds the shift term c_d d[0] x and writes the partials
-// of x . Y; 2 as 1 with the Lanczos term (- gamma q2) and the scale.
+// of x . Y; 2 as 1 with the Lanczos term (- gamma q2) and the scale; 3 as 1 with
+// a diagonal read per element, or (x nullptr) Y scaled by it.
 template <int TF, int TV, int EM>
 __global__ void __launch_bounds__(kSlabThreads, 1)
     k_kron_tc_slab(const __grid_constant__ TcSlabParams p) {
-  constexpr bool Q2 = EM == 2, HX = EM >= 1;
+  constexpr bool Q2 = EM == 2, HX = EM >= 1, DV = EM == 3;
   constexpr int kMaxT = TF > TV ? TF : TV;
   constexpr bool kSmall = TF > 1 || TV > 1;
   constexpr uint32_t kKbBytes = (uint32_t)TV * kFsBTermBytes;  // one 64-wide k block, TV terms
@@ -1785,7 +1788,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
     const int khalf = warp >> 2;             // 32 of the 64 k (= j2) of a block; i2 half
     const uint32_t taddr =
         tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + kSlabAccCol + (uint32_t)khalf * 64u;
-    const float sc = HX ? p.dcoeff * p.d[0] : 0.0f;
+    const float sc = DV ? p.dcoeff : (HX ? p.dcoeff * p.d[0] : 0.0f);
     float v[2][32];
     auto load_s = [&](int64_t sl) {
       const float* src = p.S + sl * (int64_t)(kSlabN * kSlabN) + row;
@@ -1808,21 +1811,30 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
       const float gam = Q2 ? (float)p.gamma[r] : 0.0f;
       const float srr = (HX && p.scale) ? (float)p.scale[r] : 1.0f;
       const int64_t i0 = sl * (int64_t)(kSlabN * kSlabN) + (int64_t)(khalf * 64) * kSlabN + row;
-      constexpr int kBlk = 16;
+      // the diagonal's entries of this slab (EM 3)
+      const float* dp = DV ? p.d + (sl - r * p.slabs_per_rhs) * (int64_t)(kSlabN * kSlabN) +
+                                 (int64_t)(khalf * 64) * kSlabN + row
+                           : nullptr;
+      constexpr int kBlk = DV ? 8 : 16;
       float part = 0.0f;
 #pragma unroll
       for (int blk = 0; blk < 64 / kBlk; ++blk) {
-        float xv[kBlk], qv[Q2 ? kBlk : 1];
+        float xv[kBlk], qv[Q2 ? kBlk : 1], dv[DV ? kBlk : 1];
 #pragma unroll
         for (int c = 0; c < kBlk; ++c) {
           const int64_t o = i0 + (int64_t)(blk * kBlk + c) * kSlabN;
-          xv[c] = HX ? __ldg(p.x + o) : 0.0f;
+          xv[c] = (HX && (!DV || p.x)) ? __ldg(p.x + o) : 0.0f;
+          if (DV) dv[c] = __ldg(dp + (int64_t)(blk * kBlk + c) * kSlabN);
           if (Q2) qv[c] = gam != 0.0f ? __ldg(p.q2 + o) : 0.0f;
         }
 #pragma unroll
         for (int c = 0; c < kBlk; ++c) {
           const int cc = blk * kBlk + c;
-          float y = HX ? srr * fmaf(sc, xv[c], p.coeff * a[cc]) : p.coeff * a[cc];
+          float y;
+          if (DV)
+            y = p.x ? fmaf(sc * dv[c], xv[c], p.coeff * a[cc]) : p.coeff * a[cc] * dv[c];
+          else
+            y = HX ? srr * fmaf(sc, xv[c], p.coeff * a[cc]) : p.coeff * a[cc];
           if (Q2) y = fmaf(-gam, qv[c], y);
           if (HX) part = fmaf(y, xv[c], part);
           p.Y[i0 + (int64_t)cc * kSlabN] = y;
@@ -2539,7 +2551,8 @@ static SlabKernel slab_kernel(int tf, int tv, int em) {
 #define COLA_SLAB_ROW(a, e) \
   {k_kron_tc_slab<a, 1, e>, k_kron_tc_slab<a, 2, e>, k_kron_tc_slab<a, 3, e>}
 #define COLA_SLAB_EM(e) {COLA_SLAB_ROW(1, e), COLA_SLAB_ROW(2, e), COLA_SLAB_ROW(3, e)}
-  static const SlabKernel tab[3][3][3] = {COLA_SLAB_EM(0), COLA_SLAB_EM(1), COLA_SLAB_EM(2)};
+  static const SlabKernel tab[4][3][3] = {COLA_SLAB_EM(0), COLA_SLAB_EM(1), COLA_SLAB_EM(2),
+                                          COLA_SLAB_EM(3)};
 #undef COLA_SLAB_EM
 #undef COLA_SLAB_ROW
   return tab[em][tf - 1][tv - 1];
@@ -2680,7 +2693,7 @@ static int64_t kron_tc_run(Ctx* c, const cola_linop* op, const float* X, float* 
         for (int b = 1; b <= 3; ++b) {
           COLA_CUDA(cudaFuncSetAttribute(fs_kernel(a, b),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
-          for (int em = 0; em < 3; ++em)
+          for (int em = 0; em < 4; ++em)
             COLA_CUDA(cudaFuncSetAttribute(slab_kernel(a, b, em),
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)slab_smem(a, b)));
@@ -2728,20 +2741,23 @@ static bool slab_ok(const cola_linop* kron) {
   return f1->rows == f1->cols && f1->rows <= kTileM;
 }
 
-// Steps 2 and 3 of the MVM of c_k Kron + c_d d[0] I from the slab-major first
-// step output T1: Y = c_k (K_2 (x) K_3 per slab) + c_d d[0] x [- gamma q2] and
-// the partials of x . Y.  Returns the slabs per right-hand side (K_1's side).
+// Steps 2 and 3 of the MVM of c_k Kron + c_d d[0] I (dstride 0; c_d Diag(d) else,
+// and d (.) (c_k Kron) without x) from the slab-major first step output T1: Y =
+// c_k (K_2 (x) K_3 per slab) + c_d d x [- gamma q2] and the partials of x . Y; tr:
+// the transposed factors.  Returns the slabs per right-hand side (K_1's side).
 static int64_t slab_launch(Ctx* c, const cola_linop* kron, const float* T1, float* Y,
                            const float* x, const float* q2, const double* gamma, const float* d,
                            float coeff, float dcoeff, double* dot, int64_t R,
-                           const double* scale = nullptr, int rev = 0) {
+                           const double* scale = nullptr, int rev = 0, int64_t dstride = 0,
+                           bool tr = false) {
   const int tf = (int)kron->derived.at(200).bytes;
   const int tv = std::max(1, std::min(3, c->split_vector_terms));
+  const int key = 100 + (tr ? 10 : 0) + tf;
   TcSlabParams sp{};
   sp.rev = rev;
   sp.S = T1;
-  sp.img2 = (const uint16_t*)kron->kids[1]->derived.at(100 + tf).p;
-  sp.img3 = (const uint16_t*)kron->kids[2]->derived.at(100 + tf).p;
+  sp.img2 = (const uint16_t*)kron->kids[1]->derived.at(key).p;
+  sp.img3 = (const uint16_t*)kron->kids[2]->derived.at(key).p;
   sp.img_rows2 = make_plan(kSlabN, kSlabN, tf, tv).img_rows;
   sp.img_rows3 = sp.img_rows2;
   sp.Y = Y;
@@ -2758,7 +2774,7 @@ static int64_t slab_launch(Ctx* c, const cola_linop* kron, const float* T1, floa
   sp.dot = dot;
   sp.err = tc_errflag(c);
   const int grid = (int)std::min<int64_t>(sp.nslab, c->num_sms);
-  const int em = q2 ? 2 : (x ? 1 : 0);
+  const int em = q2 ? 2 : (d && dstride ? 3 : (x ? 1 : 0));
   launch_pdl(slab_kernel(tf, tv, em), dim3(grid), dim3(kSlabThreads),
              slab_smem(tf, tv), c->s, sp);
   c->count_launch();
@@ -2768,22 +2784,36 @@ static int64_t slab_launch(Ctx* c, const cola_linop* kron, const float* T1, floa
 
 // A Kronecker product of the slab shape (see slab_ok) runs as the first mode
 // step (slab-major output) and the slab kernel (steps 2 and 3 on chip); other
-// shapes, Y = coeff K X + beta Y with beta != 0 and transposes take the d mode
-// steps.
+// shapes and Y = coeff K X + beta Y with beta != 0 take the d mode steps.
 template <>
 void kron_tc_apply<float>(Ctx* c, const cola_linop* op, const float* X, float* Y, int64_t R,
                           double coeff, double beta, int depth, bool tr) {
-  if (!tr && beta == 0.0 && slab_ok(op) && op->derived.count(200)) {
+  if (beta == 0.0 && slab_ok(op) && op->derived.count(200)) {
     float* T1 = (float*)c->ws.get(depth_name("kslab", depth, 0), 4 * (size_t)op->cols * R);
     TcFusion f1;
     f1.out_trans = 1;
     f1.nsteps = 1;
-    kron_tc_run(c, op, X, T1, R, 1.0, 0.0, depth, false, f1);
-    slab_launch(c, op, T1, Y, nullptr, nullptr, nullptr, nullptr, (float)coeff, 0.0f, nullptr,
-                R);
+    kron_tc_run(c, op, X, T1, R, 1.0, 0.0, depth, tr, f1);
+    slab_launch(c, op, T1, Y, nullptr, nullptr, nullptr, nullptr, (float)coeff, 0.0f, nullptr, R,
+                nullptr, 0, 0, tr);
     return;
   }
   kron_tc_run(c, op, X, Y, R, coeff, beta, depth, tr, TcFusion{});
+}
+
+// Y = s (.) (Kron X) with s of one vector's length; false (nothing launched) when
+// the product does not run on the slab kernel.
+bool kron_tc_scaled_apply(Ctx* c, const cola_linop* kron, const float* s, const float* X,
+                          float* Y, int64_t R, int depth) {
+  if (kron->kids.size() < 2 || !tc_supported(kron) || !kron->derived.count(200) || !slab_ok(kron))
+    return false;
+  float* T1 = (float*)c->ws.get(depth_name("kslab", depth, 0), 4 * (size_t)kron->cols * R);
+  TcFusion f1;
+  f1.out_trans = 1;
+  f1.nsteps = 1;
+  kron_tc_run(c, kron, X, T1, R, 1.0, 0.0, depth, false, f1);
+  slab_launch(c, kron, T1, Y, nullptr, nullptr, nullptr, s, 1.0f, 0.0f, nullptr, R, nullptr, 0, 1);
+  return true;
 }
 
 // Y = (c_k Kron + c_d Diag(d)) X: as kron_tc_apply with the diagonal term in the
@@ -2792,14 +2822,14 @@ void kron_tc_apply<float>(Ctx* c, const cola_linop* op, const float* X, float* Y
 bool kron_tc_shift_apply(Ctx* c, const cola_linop* kron, const cola_linop* dg, const float* X,
                          float* Y, int64_t R, double ck, double cd, int depth) {
   if (kron->kids.size() < 2 || !tc_supported(kron) || !kron->derived.count(200)) return false;
-  if (slab_ok(kron) && dg->stride == 0) {
+  if (slab_ok(kron)) {
     float* T1 = (float*)c->ws.get(depth_name("kslab", depth, 0), 4 * (size_t)kron->cols * R);
     TcFusion f1;
     f1.out_trans = 1;
     f1.nsteps = 1;
     kron_tc_run(c, kron, X, T1, R, 1.0, 0.0, depth, false, f1);
     slab_launch(c, kron, T1, Y, X, nullptr, nullptr, leaf_ptr<float>(dg), (float)ck, (float)cd,
-                nullptr, R);
+                nullptr, R, nullptr, 0, dg->stride);
     return true;
   }
   TcFusion fu;
@@ -2830,7 +2860,7 @@ int64_t kron_tc_cg_mvm(Ctx* c, const cola_linop* op, const float* z, const doubl
   const cola_linop* dg = op->kids[id];
   if (kron->kids.size() < 2 || !tc_supported(kron)) return 0;
   if (kron->derived.find(200) == kron->derived.end()) return 0;
-  if (slab_ok(kron) && dg->stride == 0) {
+  if (slab_ok(kron)) {
     // first mode step: p = z + beta p, written, and the slab-major T1; then
     // steps 2 and 3 on chip with the shift term and the p . Ap partials
     float* T1 = (float*)c->ws.get(depth_name("kslab", depth, 0), 4 * (size_t)kron->cols * R);
@@ -2846,7 +2876,7 @@ int64_t kron_tc_cg_mvm(Ctx* c, const cola_linop* op, const float* z, const doubl
     kron_tc_run(c, kron, p_old, T1, R, 1.0, 0.0, depth, false, f1);
     return slab_launch(c, kron, T1, Ap, p_new, nullptr, nullptr, leaf_ptr<float>(dg),
                        (float)op->coeffs[ik], (float)op->coeffs[id], tile_dot, R, nullptr,
-                       !rev);
+                       !rev, dg->stride);
   }
   TcFusion fu;
   fu.pro_z = z;

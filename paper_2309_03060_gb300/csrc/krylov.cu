@@ -676,9 +676,11 @@ __global__ void k_lz_b(int64_t n, T* w, const T* q, const double* a_cur, int nbl
 // GEMMs, whose one-row products ran 4096 multiply-adds in sequence.
 constexpr int kGsChunk = 512, kGsTile = 256;
 
+// Stage 0 also sums alpha_j = q . w from k_lz_a's partials (hin, one per chunk
+// block) and records it (block 0 of each vector).
 template <typename T, int STAGE>
 __global__ void __launch_bounds__(256) k_lz_gs(int64_t N, T* w, const T* q, T* Q, int cnt, int m,
-                                               const double* a_cur, const double* hin,
+                                               LzState* st, double* alpha, const double* hin,
                                                double* hout) {
   __shared__ T xs[kGsChunk];
   __shared__ T hs[kGsTile];
@@ -690,7 +692,16 @@ __global__ void __launch_bounds__(256) k_lz_gs(int64_t N, T* w, const T* q, T* Q
   T* Qv = Q + v * (int64_t)m * N;
   const int64_t step = (int64_t)nb * kGsChunk;
   if (STAGE == 0) {
-    const T a = (T)a_cur[v];
+    double as = 0.0;
+    for (int k = lane; k < nb; k += 32) as += hin[v * nb + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) as += __shfl_xor_sync(0xffffffffu, as, o);
+    const bool live = st[v].active != 0;
+    const T a = live ? (T)as : T(0);
+    if (b == 0 && tid == 0 && live) {
+      alpha[v * m + cnt - 1] = as;
+      st[v].amax = fmax(st[v].amax, fabs(as));
+    }
     for (int64_t e0 = (int64_t)b * kGsChunk; e0 < N; e0 += step)
       for (int64_t e = e0 + tid; e < N && e < e0 + kGsChunk; e += 256) {
         const T qe = q[v * N + e];
@@ -712,10 +723,21 @@ __global__ void __launch_bounds__(256) k_lz_gs(int64_t N, T* w, const T* q, T* Q
       for (int64_t e0 = (int64_t)b * kGsChunk; e0 < N; e0 += step)
         for (int64_t e = e0 + tid; e < N && e < e0 + kGsChunk; e += 256) {
           const T* qp = Qv + (int64_t)i0 * N + e;
-          T x = wv[e];
-#pragma unroll 4
-          for (int i = 0; i < ni; ++i) x = fma(-hs[i], qp[(int64_t)i * N], x);
-          wv[e] = x;
+          // two chains, eight loads in flight
+          T x = wv[e], x2 = T(0);
+          int i = 0;
+          for (; i + 8 <= ni; i += 8) {
+            T qv[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) qv[u] = qp[(int64_t)(i + u) * N];
+#pragma unroll
+            for (int u = 0; u < 8; u += 2) {
+              x = fma(-hs[i + u], qv[u], x);
+              x2 = fma(-hs[i + u + 1], qv[u + 1], x2);
+            }
+          }
+          for (; i < ni; ++i) x = fma(-hs[i], qp[(int64_t)i * N], x);
+          wv[e] = x + x2;
         }
     }
   }
@@ -740,8 +762,16 @@ __global__ void __launch_bounds__(256) k_lz_gs(int64_t N, T* w, const T* q, T* Q
       for (int i = warp; i < ni; i += 8) {
         const T* qp = Qv + (int64_t)(i0 + i) * N + e0;
         T f = T(0);
-#pragma unroll 4
-        for (int e = lane; e < len; e += 32) f = fma(qp[e], xs[e], f);
+        if (len == kGsChunk) {  // all 16 loads in flight, four chains
+          T qv[kGsChunk / 32], g[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+          for (int u = 0; u < kGsChunk / 32; ++u) qv[u] = qp[lane + 32 * u];
+#pragma unroll
+          for (int u = 0; u < kGsChunk / 32; ++u) g[u & 3] = fma(qv[u], xs[lane + 32 * u], g[u & 3]);
+          f = (g[0] + g[1]) + (g[2] + g[3]);
+        } else {
+          for (int e = lane; e < len; e += 32) f = fma(qp[e], xs[e], f);
+        }
         double t = (double)f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -753,10 +783,16 @@ __global__ void __launch_bounds__(256) k_lz_gs(int64_t N, T* w, const T* q, T* Q
   }
 }
 
+// nparts > 0: nrm2 holds that many partials per vector, summed here in order.
 __global__ void k_lz_beta(LzState* st, const double* nrm2, int64_t nv, int j, int m, double eps,
-                          double* beta, double* b_cur) {
+                          double* beta, double* b_cur, int nparts = 0) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= nv) return;
+  double n2 = 0.0;
+  if (nparts > 0)
+    for (int k = 0; k < nparts; ++k) n2 += nrm2[v * nparts + k];
+  else
+    n2 = nrm2[v];
   LzState& s = st[v];
   b_cur[v] = 0.0;
   if (!s.active) return;
@@ -765,7 +801,7 @@ __global__ void k_lz_beta(LzState* st, const double* nrm2, int64_t nv, int j, in
     s.m_eff = m;
     return;
   }
-  const double b = sqrt(fmax(nrm2[v], 0.0));
+  const double b = sqrt(fmax(n2, 0.0));
   if (!(b > eps * s.amax)) {
     s.active = 0;
     s.m_eff = j + 1;
@@ -1804,24 +1840,27 @@ static void lanczos_run(Ctx* c, cola_linop* op, const T* Q0, int64_t nv, int m, 
   const double eps = (prec == COLA_PREC_F64) ? 1e-10 : 1e-6;
   for (int j = 0; j < m; ++j) {
     apply<T>(c, op, q, w, nv, 1.0, 0.0, 1, false, prec);
-    k_lz_a<T><<<rows_grid(N, nv, nblk), 256, 0, c->s>>>(N, w, qprev, q, st, nblk, part);
-    c->count_launch();
-    k_lz_alpha<<<(unsigned)nv, 256, 0, c->s>>>(st, part, nblk, nv, j, m, alpha, a_cur);
+    const int ab = reorth ? gsb : nblk;
+    k_lz_a<T><<<rows_grid(N, nv, ab), 256, 0, c->s>>>(N, w, qprev, q, st, ab,
+                                                       reorth ? gs1 : part);
     c->count_launch();
     if (reorth) {
       const dim3 g((unsigned)gsb, (unsigned)nv);
-      k_lz_gs<T, 0><<<g, 256, 0, c->s>>>(N, w, q, Qall, j + 1, m, a_cur, nullptr, gs1);
-      k_lz_gs<T, 1><<<g, 256, 0, c->s>>>(N, w, nullptr, Qall, j + 1, m, nullptr, gs1, gs2);
-      k_lz_gs<T, 2><<<g, 256, 0, c->s>>>(N, w, nullptr, Qall, j + 1, m, nullptr, gs2, gs1);
+      k_lz_gs<T, 0><<<g, 256, 0, c->s>>>(N, w, q, Qall, j + 1, m, st, alpha, gs1, gs2);
+      k_lz_gs<T, 1><<<g, 256, 0, c->s>>>(N, w, nullptr, Qall, j + 1, m, nullptr, nullptr, gs2,
+                                         gs1);
+      k_lz_gs<T, 2><<<g, 256, 0, c->s>>>(N, w, nullptr, Qall, j + 1, m, nullptr, nullptr, gs1,
+                                         gs2);
       for (int k = 0; k < 3; ++k) c->count_launch();
-      dot_final(c, gs1, gsb, nv, nrm2);
     } else {
+      k_lz_alpha<<<(unsigned)nv, 256, 0, c->s>>>(st, part, nblk, nv, j, m, alpha, a_cur);
+      c->count_launch();
       k_lz_b<T><<<rows_grid(N, nv, nblk), 256, 0, c->s>>>(N, w, q, a_cur, nblk, part);
       c->count_launch();
       dot_final(c, part, nblk, nv, nrm2);
     }
-    k_lz_beta<<<(unsigned)((nv + 127) / 128), 128, 0, c->s>>>(st, nrm2, nv, j, m, eps, beta,
-                                                             b_cur);
+    k_lz_beta<<<(unsigned)((nv + 127) / 128), 128, 0, c->s>>>(
+        st, reorth ? gs2 : nrm2, nv, j, m, eps, beta, b_cur, reorth ? gsb : 0);
     c->count_launch();
     k_lz_next<T><<<dim3(ew_blocks(N), (unsigned)nv), 256, 0, c->s>>>(N, w, b_cur);
     c->count_launch();

@@ -391,6 +391,10 @@ constexpr int kBatchChunkCap = 128;
 
 static unsigned small_grid(int64_t n) { return (unsigned)std::max<int64_t>(1, (n + 127) / 128); }
 
+// Most bytes of factor digit images a batched solve keeps (the 512-system batch
+// with sides 16 .. 256 takes 0.5 GB).
+static constexpr size_t kF64ImageCap = (size_t)4 << 30;
+
 cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
                             const void* const* Bin, void* const* Xout, const int64_t* nrhs,
                             const cola_cg_opts& o, cola_cg_info* info, bool* handled) {
@@ -554,10 +558,82 @@ cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
     }
   };
 
+  auto residual_norms = [&](const DevSeg& dseg) {
+    k_seg_dot64<<<dseg.grid, 256, 0, c->s>>>(dseg.blocks, dseg.nblk, r64, r64, part_rr);
+    c->count_launch();
+    k_seg_sum<<<small_grid(G), 128, 0, c->s>>>(dseg.seg_list, dseg.nseg, dseg.seg_b0,
+                                               dseg.seg_nb, part_rr, rr64);
+    c->count_launch();
+  };
+
+  // The FP64 residual products run as digit products on the tensor cores
+  // (kron_f64.cu) where that is faster: steps of 64 vectors x 128 outputs x 128 k
+  // spread over the SMs at 15 us each plus 40 us of launches and fill, against
+  // 0.55e6 multiply-adds per us in 32 x 32 tiles on the FP64 units (the rule of a
+  // single product, f64_tc_pays, summed over the problems).  Measured on 64 systems
+  // with sides 16 .. 256: 153 us a product against 788 us.
+  auto f64_gain = [&](auto&& counted) {
+    double steps = 0.0, fma = 0.0;
+    bool fits = true;
+    for (int s = 0; s < nsys; ++s) {
+      if (!counted(s)) continue;
+      const BatchSys& b = sys[s];
+      auto add = [&](int64_t rest, int64_t n) {
+        steps += (double)((rest + 63) / 64 * ((n + 127) / 128) * ((n + 127) / 128) * b.R);
+        fma += (double)((rest + 31) / 32 * 32) * (double)((n + 31) / 32 * 32) * (double)(n * b.R);
+      };
+      add(b.n2, b.n1);
+      add(b.n1, b.n2);
+      fits = fits && b.N < (int64_t)1 << 30;  // 32-bit indices within a vector
+    }
+    if (!fits || steps >= 1e9) return -1.0;
+    return (20.0 + fma / 0.55e6) - (40.0 + 15.0 * steps / c->num_sms);
+  };
+  const double gain_us = f64_gain([](int) { return true; });
+  // Digit images of every factor, made once per solve at 2.5 us a factor: only if
+  // the first residual wins that back (every solve computes two or more), and none
+  // when they would take more than kF64ImageCap bytes or do not fit the device.
+  std::vector<size_t> img1(nsys), img2(nsys);
+  char* f64img = nullptr;
+  if (gain_us > 5.0 * nsys) {
+    size_t bytes = 0;
+    for (int s = 0; s < nsys; ++s) {
+      img1[s] = bytes;
+      bytes += f64_image_bytes(sys[s].n1, sys[s].n1);
+      img2[s] = bytes;
+      bytes += f64_image_bytes(sys[s].n2, sys[s].n2);
+    }
+    if (bytes <= kF64ImageCap) f64img = (char*)ws.try_get("bcg.f64img", bytes);
+  }
+  if (f64img)
+    for (int s = 0; s < nsys; ++s) {
+      const BatchSys& b = sys[s];
+      f64_factor_image(c, leaf_ptr<double>(b.f1), b.n1, 1, (int)b.n1, (int)b.n1, f64img + img1[s]);
+      f64_factor_image(c, leaf_ptr<double>(b.f2), b.n2, 1, (int)b.n2, (int)b.n2, f64img + img2[s]);
+    }
+
   // FP64 true residual r64 = b64 - A x64 for the systems in `which`
   auto residual64 = [&](const std::vector<char>& which, const DevSeg& dseg) {
     k_seg_resid_init<<<dseg.grid, 256, 0, c->s>>>(dseg.blocks, dseg.nblk, shift, b64, x64, r64);
     c->count_launch();
+    if (f64img && f64_gain([&](int s) { return which[s] != 0; }) > 0.0) {
+      // step 1: T[rest = n2][i1] = sum_j X[j1][rest] K1[i1][j1]; step 2: r[rest = n1][i2]
+      // -= ck sum_j T[j2][rest] K2[i2][j2]
+      std::vector<F64Batch> t1, t2;
+      for (int s = 0; s < nsys; ++s) {
+        if (!which[s]) continue;
+        const BatchSys& b = sys[s];
+        t1.push_back(F64Batch{x64 + b.off, T64 + b.off, leaf_ptr<double>(b.f1), f64img + img1[s],
+                              (int)b.n2, (int)b.n1, (int)b.n1, b.R, b.N, b.N, 1.0, 0.0});
+        t2.push_back(F64Batch{T64 + b.off, r64 + b.off, leaf_ptr<double>(b.f2),
+                              f64img + img2[s], (int)b.n1, (int)b.n2, (int)b.n2, b.R, b.N, b.N,
+                              -b.ck, 1.0});
+      }
+      f64_tc_batch(c, t1, "bcg.t1");
+      f64_tc_batch(c, t2, "bcg.t2");
+      residual_norms(dseg);
+      return;
+    }
     std::vector<GemmDesc<double>> g1, g2;
     int64_t mm = 1, nn = 1;
     for (int s = 0; s < nsys; ++s) {
@@ -590,11 +666,7 @@ cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
       gemm_grouped<double>(c, d2, cnt, mm, nn);
       COLA_CUDA(cudaStreamSynchronize(c->s));  // host descriptor vectors go out of scope
     }
-    k_seg_dot64<<<dseg.grid, 256, 0, c->s>>>(dseg.blocks, dseg.nblk, r64, r64, part_rr);
-    c->count_launch();
-    k_seg_sum<<<small_grid(G), 128, 0, c->s>>>(dseg.seg_list, dseg.nseg, dseg.seg_b0,
-                                               dseg.seg_nb, part_rr, rr64);
-    c->count_launch();
+    residual_norms(dseg);
   };
 
   // ---------------------------------------------------------------- set-up

@@ -56,6 +56,7 @@ struct Workspace {
   std::map<std::string, Buf> bufs;
   uint64_t generation = 0;  // bumps whenever any buffer moves (graphs key on it)
   void* get(const std::string& name, size_t bytes);
+  void* try_get(const std::string& name, size_t bytes);  // nullptr when it does not fit
   void release_all();
 };
 
@@ -203,6 +204,24 @@ void bilinear(Ctx* c, const cola_linop* op, const T* Uw, const T* X, int64_t R, 
               const std::vector<void*>& grads, int& leaf_index, int depth);
 
 void collect_leaves(const cola_linop* op, std::vector<const cola_linop*>& out);
+
+// Batches of FP64 mode steps over prepared factor images (kron_f64.cu): the
+// bytes and the making of one factor's image (256-byte aligned memory), and one
+// launch over a list of problems, each as f64_tc_mode_step with the factor F
+// row-major n_out x n_in.  Synchronises the stream.
+size_t f64_image_bytes(int64_t n_out, int64_t n_in);
+void f64_factor_image(Ctx* c, const double* F, int64_t f_i, int64_t f_j, int n_out, int n_in,
+                      void* mem);
+struct F64Batch {
+  const double* X;
+  double* Y;
+  const double* F;
+  const void* image;
+  int rest, n_out, n_in;
+  int64_t R, size_in, size_out;
+  double alpha, beta;
+};
+void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag);
 
 // ------------------------------------------------------------- kernels API
 // Diagonal term of a product's epilogue: C += coeff d (.) x, x laid out as C

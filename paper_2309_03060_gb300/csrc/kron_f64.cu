@@ -44,6 +44,8 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <string>
+#include <vector>
 
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -76,8 +78,35 @@ struct F64Params {
   int rest, tiles_m, ntiles, n_in, n_out, nchunks, kchunks;
   double alpha, beta;
   int has_alpha, has_beta;  // alpha != 1, beta != 0 (a compare is an FP64-pipe instruction)
+};
+
+// Launch-wide settings.
+struct F64Launch {
   int* err;
   uint64_t stall_ns;
+};
+
+// Where a tile's parameters come from: one problem by value, or a device table
+// of problems (tile -> problem, first tile of each).
+struct F64One {
+  F64Params p;
+  __device__ __forceinline__ int count() const { return p.ntiles; }
+  __device__ __forceinline__ const F64Params& get(int t, int& lt) const {
+    lt = t;
+    return p;
+  }
+};
+struct F64Tab {
+  const F64Params* probs;
+  const int* tile_prob;
+  const int* first;
+  int ntiles;
+  __device__ __forceinline__ int count() const { return ntiles; }
+  __device__ __forceinline__ const F64Params& get(int t, int& lt) const {
+    const int i = __ldg(tile_prob + t);
+    lt = t - __ldg(first + i);
+    return probs[i];
+  }
 };
 
 // Magnitude key of FP64 entries: the largest high word without the sign, or 1
@@ -288,8 +317,9 @@ __device__ __forceinline__ void issue_group(uint32_t tmem, uint64_t ad, uint64_t
   }
 }
 
+template <class Src>
 __global__ void __launch_bounds__(kThreadsF64, 1)
-    k_kron_f64_tc(const __grid_constant__ F64Params p) {
+    k_kron_f64_tc(const __grid_constant__ Src src, const F64Launch L) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* bdig = base;
@@ -339,9 +369,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int mine = (p.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int nsteps = (int)blockIdx.x < p.ntiles ? mine * p.kchunks : 0;
-  const int kb_last = (p.n_in - (p.kchunks - 1) * kKc + 63) / 64;  // k blocks, last chunk
+  const int ntiles = src.count();
 
   if (warp == kLoadWarp) {
     // -------------------------------------------------- factor digit copies
@@ -349,19 +377,22 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       int s = 0;
       uint32_t ph = 0, issued = 0, issued_ph = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x) {
-        const int nc = tile % p.nchunks;
-        for (int kc = 0; kc < p.kchunks && ok; ++kc) {
-          const uint32_t bytes = (kc == p.kchunks - 1 ? kb_last : 2) * (kADig / 2);
-          const unsigned char* src = (const unsigned char*)p.img +
-                                     ((int64_t)nc * p.kchunks + kc) * (int64_t)(kDg * kADig);
+      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        int lt;
+        const F64Params& p = src.get(tile, lt);
+        const int kchunks = p.kchunks, nc = lt % p.nchunks;
+        const int kb_last = (p.n_in - (kchunks - 1) * kKc + 63) / 64;  // k blocks, last chunk
+        const unsigned char* img =
+            (const unsigned char*)p.img + (int64_t)nc * kchunks * (int64_t)(kDg * kADig);
+        for (int kc = 0; kc < kchunks && ok; ++kc, img += kDg * kADig) {
+          const uint32_t bytes = (kc == kchunks - 1 ? kb_last : 2) * (kADig / 2);
           for (int a = 0; a < kDg; ++a) {
-            if (!mbar_wait(&aempty[s], ph ^ 1u, abort_flag, p.err)) {
+            if (!mbar_wait(&aempty[s], ph ^ 1u, abort_flag, L.err)) {
               ok = false;
               break;
             }
             mbar_arrive_expect_tx(&afull[s], bytes);
-            bulk_g2s(adig + s * kADig, src + a * kADig, bytes, &afull[s]);
+            bulk_g2s(adig + s * kADig, img + a * kADig, bytes, &afull[s]);
             issued |= 1u << s;
             issued_ph = (issued_ph & ~(1u << s)) | (ph << s);
             if (++s == kABufs) {
@@ -373,7 +404,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       }
       // the latest copy into each buffer is the only one that can be in flight
       for (int b = 0; b < kABufs; ++b)
-        if (issued & (1u << b)) mbar_wait_own(&afull[b], (issued_ph >> b) & 1u, p.err);
+        if (issued & (1u << b)) mbar_wait_own(&afull[b], (issued_ph >> b) & 1u, L.err);
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
@@ -382,21 +413,24 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     const uint32_t elect = elect_one();
     constexpr uint32_t idesc = idesc_f16(kOut, kVec);
     bool ok = true;
-    if (p.stall_ns)
-      ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, p.err, p.stall_ns));
+    if (L.stall_ns)
+      ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, L.err, L.stall_ns));
     const uint64_t adesc = sw128_desc(smem_u32(adig)), bdesc = sw128_desc(smem_u32(bdig));
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
     int s = 0;
     uint32_t ph = 0, sph = 0;
-    for (int tile = blockIdx.x; tile < p.ntiles && ok; tile += gridDim.x) {
-      for (int kc = 0; kc < p.kchunks && ok; ++kc, sph ^= 1u) {
-        const int kleft = p.n_in - kc * kKc;
+    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      int lt;
+      const F64Params& p = src.get(tile, lt);
+      const int kchunks = p.kchunks, n_in = p.n_in;
+      for (int kc = 0; kc < kchunks && ok; ++kc, sph ^= 1u) {
+        const int kleft = n_in - kc * kKc;
         const int ksteps = kleft >= kKc ? 8 : (kleft + 15) / 16;
-        ok = mbar_wait_warp(ready, sph, abort_flag, p.err);
+        ok = mbar_wait_warp(ready, sph, abort_flag, L.err);
         if (!ok) break;
         tc_fence_after();
         for (int a = 0; a < kDg; ++a) {
-          ok = mbar_wait_warp(&afull[s], ph, abort_flag, p.err);
+          ok = mbar_wait_warp(&afull[s], ph, abort_flag, L.err);
           if (!ok) break;
           tc_fence_after();
           // descriptors advance by address / 16: 2 per 16-wide k step
@@ -416,14 +450,14 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     }
     // the elected lane's commit covers every MMA it issued
     mma_commit_one(drain, elect);
-    if (elect) mbar_wait_own(drain, 0, p.err);
+    if (elect) mbar_wait_own(drain, 0, L.err);
     __syncwarp();
   } else if (warp < kConvWarps) {
     // ----------------------------------------------------------- converters
     // vector n of the tile, 8-entry k runs at k = 8 oct + 32 h, h < 4
     const int n = (warp & 1) * 32 + lane, oct = warp >> 1;
     unsigned long long u[32];
-    auto load = [&](const F64Step& s) {
+    auto load = [&](const F64Params& p, const F64Step& s) {
       const int m = s.m0 + n;
       const double* x = p.X + s.r * p.size_in + m;
       const int k0 = s.kc * kKc + oct * 8;
@@ -444,9 +478,15 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       }
     };
     int tile = blockIdx.x, kc = 0;
-    if (nsteps > 0) load(step_of(p, tile, 0));
+    if (tile < ntiles) {
+      int lt;
+      const F64Params& p = src.get(tile, lt);
+      load(p, step_of(p, lt, 0));
+    }
     bool ok = true;
-    for (int st = 0; st < nsteps; ++st) {
+    for (int st = 0; tile < ntiles; ++st) {
+      int lt;
+      const F64Params& p = src.get(tile, lt);
       const int par = st & 1;
       uint32_t xh = 0, xl = 0;
 #pragma unroll
@@ -459,7 +499,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       const int emax = key >> 20;
       const bool dig = key != 0 && has_digits(key);
       if (st > 1) {  // the drainers are done with the keys of step st - 2
-        if (ok) ok = mbar_wait(&kfree[par], (uint32_t)((st >> 1) + 1) & 1u, abort_flag, p.err);
+        if (ok) ok = mbar_wait(&kfree[par], (uint32_t)((st >> 1) + 1) & 1u, abort_flag, L.err);
         ok = __all_sync(0xffffffffu, ok);
       }
       if (oct == 0) {
@@ -480,7 +520,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       const uint32_t dph = (uint32_t)((st + 1) & 1);
 #define COLA_DIGIT(S)                                                      \
   if (st > 0) {                                                            \
-    if (ok) ok = mbar_wait(&dfull[S], dph, abort_flag, p.err);             \
+    if (ok) ok = mbar_wait(&dfull[S], dph, abort_flag, L.err);             \
     ok = __all_sync(0xffffffffu, ok);                                      \
   }                                                                        \
   put_digit<6 - S>(bdig, u, n, oct, kpad);
@@ -495,20 +535,27 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(ready);
-      if (++kc == p.kchunks) {
-        kc = 0;
-        tile += gridDim.x;
-      }
-      if (st + 1 < nsteps) load(step_of(p, tile, kc));
-      if (st + 2 < nsteps) {  // the block after it: DRAM to L2, two 128-byte lines a thread
-        const bool wrap = kc + 1 == p.kchunks;
-        const F64Step f = step_of(p, wrap ? tile + (int)gridDim.x : tile, wrap ? 0 : kc + 1);
+      const bool wrap = kc + 1 == p.kchunks;
+      tile = wrap ? tile + (int)gridDim.x : tile;
+      kc = wrap ? 0 : kc + 1;
+      if (tile < ntiles) {
+        int nlt;
+        const F64Params& q = src.get(tile, nlt);
+        load(q, step_of(q, nlt, kc));
+        // the block after it: DRAM to L2, two 128-byte lines a thread
+        const bool wrap2 = kc + 1 == q.kchunks;
+        const int t2 = wrap2 ? tile + (int)gridDim.x : tile;
+        if (t2 < ntiles) {
+          int lt2;
+          const F64Params& n2 = src.get(t2, lt2);
+          const F64Step f = step_of(n2, lt2, wrap2 ? 0 : kc + 1);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = f.kc * kKc + (tid >> 2) + 64 * h, m = f.m0 + (tid & 3) * 16;
-          if (k < p.n_in && m < p.rest)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.X + f.r * p.size_in +
-                                                           (int64_t)k * p.rest + m));
+          for (int h = 0; h < 2; ++h) {
+            const int k = f.kc * kKc + (tid >> 2) + 64 * h, m = f.m0 + (tid & 3) * 16;
+            if (k < n2.n_in && m < n2.rest)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(n2.X + f.r * n2.size_in +
+                                                             (int64_t)k * n2.rest + m));
+          }
         }
       }
     }
@@ -520,14 +567,16 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     long long acc[32];
     int tile = blockIdx.x, kc = 0;
     bool ok = true;
-    if (nsteps > 0 && lane == 0) mbar_arrive(ready);  // nothing to drain before step 0
-    for (int st = 0; st < nsteps; ++st) {
+    if (tile < ntiles && lane == 0) mbar_arrive(ready);  // nothing to drain before step 0
+    for (int st = 0; tile < ntiles; ++st) {
+      int lt;
+      const F64Params& p = src.get(tile, lt);
       const int par = st & 1;
-      const int nc = tile % p.nchunks;
+      const int nc = lt % p.nchunks;
       // the factor row's exponent, ahead of its use in the store
       const int ef = __ldg(&p.fexp[((int64_t)nc * p.kchunks + kc) * kOut + orow]);
 #define COLA_DIGIT(S)                                                      \
-  if (ok) ok = mbar_wait(&dfull[S], (uint32_t)par, abort_flag, p.err);     \
+  if (ok) ok = mbar_wait(&dfull[S], (uint32_t)par, abort_flag, L.err);     \
   ok = __all_sync(0xffffffffu, ok);                                        \
   tc_fence_after();                                                        \
   if (ok) fold<S>(taddr, acc);
@@ -541,10 +590,11 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
 #undef COLA_DIGIT
       tc_fence_before();
       __syncwarp();
-      if (lane == 0 && st + 1 < nsteps) mbar_arrive(ready);
-      if (ok) ok = mbar_wait(&kfull[par], (uint32_t)(st >> 1) & 1u, abort_flag, p.err);
+      const bool more = kc + 1 < p.kchunks || tile + (int)gridDim.x < ntiles;
+      if (lane == 0 && more) mbar_arrive(ready);
+      if (ok) ok = mbar_wait(&kfull[par], (uint32_t)(st >> 1) & 1u, abort_flag, L.err);
       ok = __all_sync(0xffffffffu, ok);
-      const F64Step cur = step_of(p, tile, kc);
+      const F64Step cur = step_of(p, lt, kc);
       const int i = nc * kOut + orow;
       const int cnt = min(32, p.rest - cur.m0 - oc0);
       if (ok && i < p.n_out && cnt > 0) {
@@ -616,6 +666,84 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
 
 }  // namespace
 
+template <class Src>
+static void f64_launch(Ctx* c, const Src& src, int ntiles) {
+  F64Launch L{tc_errflag(c), 0};
+  if (c->tc_stall_ns > 0 && !c->capturing) {
+    L.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
+    c->tc_stall_ns = 0;
+  }
+  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemF64));
+  k_kron_f64_tc<Src><<<std::min(ntiles, c->num_sms), kThreadsF64, kSmemF64, c->s>>>(src, L);
+  c->count_launch();
+  c->f64_tc_used = true;
+  COLA_CUDA(cudaGetLastError());
+}
+
+size_t f64_image_bytes(int64_t n_out, int64_t n_in) {
+  return (size_t)((n_out + kOut - 1) / kOut) * (size_t)((n_in + kKc - 1) / kKc) *
+         (kDg * kADig + kOut * 4);
+}
+
+void f64_factor_image(Ctx* c, const double* F, int64_t f_i, int64_t f_j, int n_out, int n_in,
+                      void* mem) {
+  const int nch = (n_out + kOut - 1) / kOut, kch = (n_in + kKc - 1) / kKc;
+  k_f64_digits<<<dim3(kOut, (unsigned)nch, (unsigned)kch), kKc, 0, c->s>>>(
+      F, f_i, f_j, n_out, n_in, kch, (uint16_t*)mem,
+      (int*)((char*)mem + (size_t)nch * kch * (kDg * kADig)));
+  c->count_launch();
+  COLA_CUDA(cudaGetLastError());
+}
+
+void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
+  std::vector<F64Params> hp(probs.size());
+  std::vector<int> first(probs.size()), tile_prob;
+  for (size_t i = 0; i < probs.size(); ++i) {
+    const F64Batch& b = probs[i];
+    F64Params& p = hp[i];
+    p = F64Params{};
+    p.nchunks = (b.n_out + kOut - 1) / kOut;
+    p.kchunks = (b.n_in + kKc - 1) / kKc;
+    p.tiles_m = (b.rest + kVec - 1) / kVec;
+    p.ntiles = (int)(b.R * p.tiles_m * p.nchunks);
+    p.X = b.X;
+    p.Y = b.Y;
+    p.F = b.F;
+    p.f_i = b.n_in;
+    p.f_j = 1;
+    p.img = (const uint16_t*)b.image;
+    p.fexp = (const int*)((const char*)b.image + (size_t)p.nchunks * p.kchunks * (kDg * kADig));
+    p.rest = b.rest;
+    p.n_in = b.n_in;
+    p.n_out = b.n_out;
+    p.size_in = b.size_in;
+    p.size_out = b.size_out;
+    p.alpha = b.alpha;
+    p.beta = b.beta;
+    p.has_alpha = b.alpha != 1.0;
+    p.has_beta = b.beta != 0.0;
+    first[i] = (int)tile_prob.size();
+    tile_prob.insert(tile_prob.end(), (size_t)p.ntiles, (int)i);
+  }
+  const int nt = (int)tile_prob.size(), np = (int)probs.size();
+  if (nt == 0) return;
+  const std::string t = tag;
+  F64Tab src{};
+  src.probs = (const F64Params*)c->ws.get(t + ".p", sizeof(F64Params) * np);
+  src.tile_prob = (const int*)c->ws.get(t + ".t", 4 * (size_t)nt);
+  src.first = (const int*)c->ws.get(t + ".f", 4 * (size_t)np);
+  src.ntiles = nt;
+  COLA_CUDA(cudaMemcpyAsync((void*)src.probs, hp.data(), sizeof(F64Params) * np,
+                            cudaMemcpyHostToDevice, c->s));
+  COLA_CUDA(cudaMemcpyAsync((void*)src.tile_prob, tile_prob.data(), 4 * (size_t)nt,
+                            cudaMemcpyHostToDevice, c->s));
+  COLA_CUDA(cudaMemcpyAsync((void*)src.first, first.data(), 4 * (size_t)np,
+                            cudaMemcpyHostToDevice, c->s));
+  f64_launch(c, src, nt);
+  COLA_CUDA(cudaStreamSynchronize(c->s));  // the host tables go out of scope
+}
+
 bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, const double* X,
                       int64_t size_in, const double* F, int64_t f_i, int64_t f_j, double beta,
                       double* Y, int64_t size_out, int64_t R) {
@@ -631,8 +759,9 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.ntiles = (int)(R * tiles_m * p.nchunks);
   const size_t blocks = (size_t)p.nchunks * p.kchunks;
   if (p.nchunks > 65535 || p.kchunks > 65535 || blocks > 1024) return false;
-  uint16_t* img = (uint16_t*)c->ws.get("f64.img", blocks * kDg * kADig);
-  int* fexp = (int*)c->ws.get("f64.exp", blocks * kOut * 4);
+  uint16_t* img = (uint16_t*)c->ws.try_get("f64.img", blocks * kDg * kADig);
+  int* fexp = (int*)c->ws.try_get("f64.exp", blocks * kOut * 4);
+  if (!img || !fexp) return false;
   k_f64_digits<<<dim3(kOut, (unsigned)p.nchunks, (unsigned)p.kchunks), kKc, 0, c->s>>>(
       F, f_i, f_j, n_out, n_in, p.kchunks, img, fexp);
   c->count_launch();
@@ -652,18 +781,7 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.beta = beta;
   p.has_alpha = alpha != 1.0;
   p.has_beta = beta != 0.0;
-  p.err = tc_errflag(c);
-  if (c->tc_stall_ns > 0 && !c->capturing) {
-    p.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
-    c->tc_stall_ns = 0;
-  }
-  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemF64));
-  const int grid = (int)std::min<int64_t>(p.ntiles, c->num_sms);
-  k_kron_f64_tc<<<grid, kThreadsF64, kSmemF64, c->s>>>(p);
-  c->count_launch();
-  c->f64_tc_used = true;
-  COLA_CUDA(cudaGetLastError());
+  f64_launch(c, F64One{p}, p.ntiles);
   return true;
 }
 

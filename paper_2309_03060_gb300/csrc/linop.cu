@@ -32,6 +32,12 @@ void fail(cola_status st, const char* fmt, ...) {
 
 // --------------------------------------------------------------- workspace
 void* Workspace::get(const std::string& name, size_t bytes) {
+  void* p = try_get(name, bytes);
+  if (!p) fail(COLA_ERR_OOM, "workspace '%s': cudaMalloc(%zu) failed", name.c_str(), bytes);
+  return p;
+}
+
+void* Workspace::try_get(const std::string& name, size_t bytes) {
   bytes = std::max<size_t>(bytes, 256);
   auto it = bufs.find(name);
   if (it != bufs.end() && it->second.bytes >= bytes) return it->second.p;
@@ -43,8 +49,7 @@ void* Workspace::get(const std::string& name, size_t bytes) {
   cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    fail(COLA_ERR_OOM, "workspace '%s': cudaMalloc(%zu) failed: %s", name.c_str(), bytes,
-         cudaGetErrorString(e));
+    return nullptr;
   }
   bufs[name] = Buf{p, bytes};
   ++generation;

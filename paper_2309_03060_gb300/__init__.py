@@ -65,11 +65,19 @@ class Context:
         check(lib.cola_create(int(device), C.byref(h)))
         self.handle = h
         self.device = torch.device("cuda", device)
+        self._terms = None  # split terms last handed to the library
 
     def close(self):
         if self.handle:
             check(_lib().cola_destroy(self.handle))
             self.handle = None
+
+    def _set_split_terms(self, split_terms):
+        """The library's split-term setting (kept between calls)."""
+        ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
+        if (ft, vt) != self._terms:
+            check(_lib().cola_set_split_terms(self.handle, int(ft), int(vt)))
+            self._terms = (ft, vt)
 
     def kernel_launches(self) -> int:
         n = C.c_int64()
@@ -111,6 +119,7 @@ class LinOp:
         self._keep = list(keep)
         self._seen = [t._version for t in self._keep]
         self._children = list(children)
+        self._shape = None
         if self._keep and handle:
             check(_lib().cola_linop_cache_prepared(handle, 1))
 
@@ -132,12 +141,15 @@ class LinOp:
     @handle.setter
     def handle(self, h):
         self._h = h
+        self._shape = None
 
     @property
     def shape(self):
-        r, c = C.c_int64(), C.c_int64()
-        check(_lib().cola_linop_shape(self.handle, C.byref(r), C.byref(c)))
-        return (r.value, c.value)
+        if self._shape is None:  # a node's shape never changes
+            r, c = C.c_int64(), C.c_int64()
+            check(_lib().cola_linop_shape(self.handle, C.byref(r), C.byref(c)))
+            self._shape = (r.value, c.value)
+        return self._shape
 
     def leaves(self):
         """[(kind, rows, cols)] in tree order."""
@@ -159,6 +171,7 @@ class LinOp:
         if self._h:
             check(_lib().cola_linop_release(self._h))
             self._h = None
+            self._shape = None
 
     def __del__(self):
         try:
@@ -225,8 +238,7 @@ def cola_matvec(ctx: Context, op: LinOp, X: torch.Tensor, precision: int = PREC_
     if X2.dtype != want:
         raise TypeError(f"precision {precision} needs {want} vectors")
     Y = out if out is not None else torch.empty((X2.shape[0], rows), dtype=want, device=X.device)
-    ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
-    check(_lib().cola_set_split_terms(ctx.handle, int(ft), int(vt)))
+    ctx._set_split_terms(split_terms)
     check(_lib().cola_matvec(ctx.handle, op.handle, _ptr(X2), _ptr(Y), X2.shape[0], precision,
                              _stream()))
     return Y if X.dim() == 2 else Y.reshape(-1)
@@ -379,8 +391,7 @@ def cola_lanczos(ctx: Context, op: LinOp, Q0: torch.Tensor, m: int, precision: i
     """reorth: 0 none, 1 full reorthogonalisation, 2 Householder basis;
     split_terms (MIXED) as in cola_matvec."""
     nv = Q0.shape[0]
-    ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
-    check(_lib().cola_set_split_terms(ctx.handle, int(ft), int(vt)))
+    ctx._set_split_terms(split_terms)
     alpha = torch.zeros((nv, m), dtype=torch.float64, device=Q0.device)
     beta = torch.zeros((nv, m), dtype=torch.float64, device=Q0.device)
     meff = torch.zeros(nv, dtype=torch.int32, device=Q0.device)
@@ -394,8 +405,7 @@ def cola_slq_logdet(ctx: Context, op: LinOp, nprobes: int, m: int, seed: int = 0
                     reorth: int = 0, split_terms=2):
     """Returns (logdet, std_err, per_probe tensor, clamped count); split_terms
     (MIXED) as in cola_matvec."""
-    ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
-    check(_lib().cola_set_split_terms(ctx.handle, int(ft), int(vt)))
+    ctx._set_split_terms(split_terms)
     ld, se = C.c_double(), C.c_double()
     cl = C.c_int32()
     pp = torch.empty(nprobes, dtype=torch.float64, device=ctx.device)
@@ -412,8 +422,7 @@ def cola_diag_estimate(ctx: Context, op: LinOp, nprobes: int, seed: int = 0,
     split_terms (MIXED) as in cola_matvec.  Returns (diag, trace)."""
     diag = torch.empty(op.shape[0], dtype=torch.float64, device=ctx.device)
     tr = C.c_double()
-    ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
-    check(_lib().cola_set_split_terms(ctx.handle, int(ft), int(vt)))
+    ctx._set_split_terms(split_terms)
     check(_lib().cola_diag_estimate(ctx.handle, op.handle, nprobes,
                                     C.c_uint64(seed & (2**64 - 1)), int(doubly), precision,
                                     _ptr(diag), C.byref(tr), _stream()))

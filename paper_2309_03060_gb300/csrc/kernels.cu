@@ -141,9 +141,9 @@ __global__ void __launch_bounds__(256) k_gemm(GemmP<T> g, int64_t batch0) {
 // The next k tile's loads are held in registers while the current one is
 // multiplied out of the other shared-memory buffer.  TN follows the factor's
 // side, so that a side of 97 runs 112 wide instead of 128.  Bound by the FP32
-// pipe and the shared-memory reads: 97 x 120 x 101, 5 vectors, 144 us for the
-// three modes (26 TFLOP/s of 80.5) against 288 us in the generic 128 x 128 tiles
-// that unaligned sides took before.
+// pipe and the shared-memory reads: 97 x 120 x 101, 5 vectors, 135 us for the
+// three modes (28 TFLOP/s of 80.5; 144 us with one 4-byte load per column) against
+// 288 us in the generic 128 x 128 tiles that unaligned sides took before.
 constexpr int kMfBM = 128, kMfBK = 16;
 
 __device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a,
@@ -156,11 +156,20 @@ __device__ __forceinline__ unsigned long long pack2(float v) {
   return r;
 }
 
+// Column of a thread's j-th output: groups of 4, 2 and 1 adjacent columns by the
+// binary digits of TN, so that a group is one shared-memory load.
+template <int TN>
+__device__ __forceinline__ int mode_col(int tx, int j) {
+  if (j < (TN & 12)) return 16 * (j & ~3) + 4 * tx + (j & 3);
+  if (j < (TN & 14)) return 16 * (TN & 12) + 2 * tx + (j & 1);
+  return 16 * (TN - 1) + tx;
+}
+
 template <int TN>
 __global__ void __launch_bounds__(256, 2) k_gemm_mode_f32(GemmP<float> g, int64_t batch0) {
-  constexpr int BN = 16 * TN, BNP = BN + 2;
+  constexpr int BN = 16 * TN, BNP = BN + 4;
   __shared__ __align__(16) float As[2][kMfBK][kMfBM];
-  __shared__ float Bs[2][kMfBK][BNP];
+  __shared__ __align__(16) float Bs[2][kMfBK][BNP];
   const int64_t b = batch0 + blockIdx.z;
   const int64_t m0 = (int64_t)blockIdx.x * kMfBM, n0 = (int64_t)blockIdx.y * BN;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -197,9 +206,20 @@ __global__ void __launch_bounds__(256, 2) k_gemm_mode_f32(GemmP<float> g, int64_
   auto step = [&](int buf, int kk) {
     const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][ty * 4]);
     const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][64 + ty * 4]);
+    float bv[TN];
+    const float* bs = Bs[buf][kk];
+#pragma unroll
+    for (int j = 0; j + 4 <= TN; j += 4)
+      ld4(bv + j, bs + 16 * j + 4 * tx);
+    if (TN & 2) {
+      const float2 h = *reinterpret_cast<const float2*>(bs + 16 * (TN & 12) + 2 * tx);
+      bv[TN & 12] = h.x;
+      bv[(TN & 12) + 1] = h.y;
+    }
+    if (TN & 1) bv[TN - 1] = bs[16 * (TN - 1) + tx];
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const unsigned long long bb = pack2(Bs[buf][kk][tx + 16 * j]);
+      const unsigned long long bb = pack2(bv[j]);
       fma2(acc[0][j], a0.x, bb);
       fma2(acc[1][j], a0.y, bb);
       fma2(acc[2][j], a1.x, bb);
@@ -229,7 +249,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_mode_f32(GemmP<float> g, int64_
     float* row = g.C + b * g.sC + m * g.lcm;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int64_t n = n0 + tx + 16 * j;
+      const int64_t n = n0 + mode_col<TN>(tx, j);
       if (n >= g.N) continue;
       const unsigned long long a = acc[i >> 1][j];
       float v = g.alpha * __uint_as_float((uint32_t)((i & 1) ? a >> 32 : a));

@@ -154,7 +154,8 @@ cola_status cola_linop_release(cola_linop* op);
 
 /* Y = A X for nrhs vectors (Sec. 3.1).  X is [nrhs][cols], Y is [nrhs][rows],
  * both FP64 for COLA_PREC_F64 and FP32 otherwise.  Asynchronous on stream.
- * A tensor-core kernel that gave up waiting (COLA_ERR_TIMEOUT, MIXED only) is
+ * A tensor-core kernel that gave up waiting (COLA_ERR_TIMEOUT; MIXED, and F64
+ * products large enough for the tensor cores) is
  * reported by a later call on the same context: the next cola_matvec once the
  * device has passed this one, or any call that synchronises (solves). */
 cola_status cola_matvec(cola_ctx* ctx, const cola_linop* op, const void* X, void* Y,

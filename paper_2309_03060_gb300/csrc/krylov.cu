@@ -1293,15 +1293,21 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
   if (B.kprec) chunk = std::min(chunk, kPRing);
   if (B.fused_tiles > 0) chunk = (chunk + kPRing - 1) / kPRing * kPRing;
   if (B.lr.on) chunk = (chunk + 1) / 2 * 2;  // two p buffers
+  // A solve is counted in whole chunks after its first iteration: chunk_end is
+  // the end of the chunk that iteration i (>= 1) lies in, `cap` the one where a
+  // solve stops for maxiter.
+  auto chunk_end = [&](int64_t i) { return i <= 1 ? i : 1 + (i - 1 + chunk - 1) / chunk * chunk; };
+  const int64_t cap = chunk_end(o.maxiter);
   // Without refinement the iterations after the last right-hand side stopped are
-  // lost, and nothing else depends on where a chunk ends: chunks start at 8
-  // iterations and grow (up to `chunk`) until one takes kChunkSeconds, well above
-  // the ~15 us a host check costs (2^20-point stencil + low-rank solve, 21
-  // iterations: 25 run instead of 65, 11.6 -> 5.5 ms).  Refined solves replace residuals at chunk
-  // ends and keep the fixed length.
-  int run_chunk = refine ? chunk : std::min(chunk, kPRing);
-  // the cap a solve in whole chunks would stop at
-  const int64_t cap = o.maxiter <= 1 ? o.maxiter : 1 + (o.maxiter - 1 + chunk - 1) / chunk * chunk;
+  // lost: a chunk is run in parts of 8 iterations at first and of more (up to the
+  // chunk) until one takes kChunkSeconds, well above the ~15 us a host check costs,
+  // and is left at the first part that ends with every right-hand side stopped
+  // (2^20-point stencil + low-rank solve, 21 iterations: 25 run instead of 65, 11.6
+  // -> 5.5 ms).  No part crosses the chunk's end and the iterations not run count,
+  // so that the cap, the verification and its restarts do not depend on the times
+  // measured here.  Refined solves replace residuals at chunk ends and run whole
+  // chunks.
+  int want_chunk = refine ? chunk : std::min(chunk, kPRing), run_chunk = want_chunk;
   // everything a captured kernel bakes in is part of the graph key
   auto graph_key = [&] {
     char extra[128];
@@ -1348,21 +1354,24 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
     if (iters >= cap) break;
     if (B.small.on) {
       // ends by itself when every right-hand side has stopped
-      small_cg_run<T>(c, B.small, B.r, B.x, B.p, B.invd, B.st, R,
-                      (int)std::min<int64_t>(cap - iters, kSmallChunk));
+      const int limit = (int)std::min<int64_t>(cap - iters, kSmallChunk);
+      int64_t ran = 0;
+      std::vector<int64_t> before(R);
+      for (int64_t r = 0; r < R; ++r) before[r] = hst[r].iters;
+      small_cg_run<T>(c, B.small, B.r, B.x, B.p, B.invd, B.st, R, limit);
       read_state();
       any_active = false;
-      int64_t most = 0;
       for (int64_t r = 0; r < R; ++r) {
         any_active |= hst[r].active != 0;
-        most = std::max<int64_t>(most, hst[r].iters);
+        ran = std::max<int64_t>(ran, hst[r].iters - before[r]);
       }
-      if (most <= iters) tc_check_error(c);  // no progress: the kernel gave up
-      iters = std::max(most, iters + (most <= iters ? 1 : 0));
+      if (any_active && ran < limit) tc_check_error(c);  // the kernel gave up waiting
+      iters = any_active ? iters + limit : chunk_end(iters + std::max<int64_t>(ran, 1));
       trace_line("chunk");
       continue;
     }
     const auto tc0 = std::chrono::steady_clock::now();
+    if (!refine) run_chunk = (int)std::min<int64_t>(want_chunk, chunk_end(iters + 1) - iters);
     cg_chunk<T>(c, op, B, N, R, nblk, prec, delta2, refine ? 1 : 0, run_chunk, graph_key());
     iters += run_chunk;
     read_state();
@@ -1373,7 +1382,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
       if (!refine) {
         int want = std::min(chunk, kPRing);
         while (want < chunk && want * iter_s < kChunkSeconds) want *= 2;
-        run_chunk = std::min(want, chunk);
+        want_chunk = std::min(want, chunk);
       }
     }
     trace_line("chunk");
@@ -1395,6 +1404,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
       paused |= hst[r].paused != 0;
     }
     any_active = nact > 0;
+    if (!any_active) iters = chunk_end(iters);
     const bool flag = paused || (defer ? (nflag > 0 && 2 * nflag >= nact) : nflag > 0);
     if (refine && (flag || !any_active) && updates < o.max_updates) {
       const auto tr0 = std::chrono::steady_clock::now();

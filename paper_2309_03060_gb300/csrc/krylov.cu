@@ -1127,6 +1127,7 @@ static void cg_flush_x(Ctx* c, CgBufs<T>& B, int64_t N, int64_t R, int nblk) {
 template <typename T>
 static void cg_chunk(Ctx* c, const cola_linop* op, CgBufs<T>& B, int64_t N, int64_t R, int nblk,
                      int prec, double delta2, int refine, int chunk, const std::string& key) {
+  const int cur0 = B.cur;
   auto it = c->graphs.find(key);
   if (it == c->graphs.end() || it->second.generation != c->ws.generation) {
     if (it != c->graphs.end()) {
@@ -1161,6 +1162,10 @@ static void cg_chunk(Ctx* c, const cola_linop* op, CgBufs<T>& B, int64_t N, int6
   }
   COLA_CUDA(cudaGraphLaunch(it->second.exec, c->s));
   c->launches += it->second.kernels;
+  if (B.lr.on) {  // two p buffers: an odd chunk ends on the other one
+    B.cur = (cur0 + chunk) & 1;
+    B.p = B.pp[B.cur];
+  }
 }
 
 template <typename T>
@@ -1292,7 +1297,6 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
   // chunks keep the replacements (and restarts) close behind it
   if (B.kprec) chunk = std::min(chunk, kPRing);
   if (B.fused_tiles > 0) chunk = (chunk + kPRing - 1) / kPRing * kPRing;
-  if (B.lr.on) chunk = (chunk + 1) / 2 * 2;  // two p buffers
   // A solve is counted in whole chunks after its first iteration: chunk_end is
   // the end of the chunk that iteration i (>= 1) lies in, `cap` the one where a
   // solve stops for maxiter.

@@ -53,7 +53,7 @@ def _setup(cola, path, shift=0.1):
 
 
 @pytest.mark.parametrize("path", list(PATHS))
-@pytest.mark.parametrize("maxiter,chunk", [(100, 64), (33, 40), (2, 16), (150, 24)])
+@pytest.mark.parametrize("maxiter,chunk", [(100, 64), (100, 5), (33, 40), (2, 16), (150, 24)])
 def test_capped_solve_stops_at_the_chunk_of_maxiter(path, maxiter, chunk):
     import paper_2309_03060_gb300 as cola
     ctx, op, B, P = _setup(cola, path)

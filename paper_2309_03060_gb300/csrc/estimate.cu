@@ -111,7 +111,7 @@ extern "C" cola_status cola_diag_estimate(cola_ctx* ctx, const cola_linop* op, i
       estimate<double>(ctx, op, nprobes, seed, doubly != 0, precision, acc);
     else
       estimate<float>(ctx, op, nprobes, seed, doubly != 0, precision, acc);
-    if (precision == COLA_PREC_MIXED) tc_check_error(ctx);
+    tc_check_results(ctx, precision);
     if (trace) {
       const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, 1024));
       double* part = (double*)ctx->ws.get("est.part", 8 * 1024);

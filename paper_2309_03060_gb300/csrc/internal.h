@@ -389,6 +389,9 @@ void bilinear_entry(Ctx* c, const cola_linop* op, const void* U, const void* X,
 void check_cg_args(const cola_linop* op, const cola_cg_opts* o, int64_t R);
 // Raises COLA_ERR_TIMEOUT when a tensor-core kernel gave up waiting (and clears the flag).
 void tc_check_error(Ctx* c);        // synchronises the stream
+// Before a call returns host results: tc_check_error where products of that
+// precision, or FP64 products, may have run on the tensor cores.
+void tc_check_results(Ctx* c, int prec);
 void tc_check_error_async(Ctx* c);  // reports an earlier call's timeout, queues a check
 void tc_check_earlier(Ctx* c, cudaStream_t user);  // FP64 products of earlier calls
 int* tc_errflag(Ctx* c);            // device flag the tensor-core kernels raise

@@ -2155,6 +2155,10 @@ void tc_check_error(Ctx* c) {
   }
 }
 
+void tc_check_results(Ctx* c, int prec) {
+  if (prec == COLA_PREC_MIXED || c->f64_tc_used) tc_check_error(c);
+}
+
 // The device flag is only cleared when a timeout is reported, so a copy taken
 // at any later point still shows it.  One copy is in flight at a time.
 // queue = false: only reads a copy that has arrived.

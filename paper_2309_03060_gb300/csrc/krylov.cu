@@ -1482,7 +1482,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
     apply<T>(c, op, B.x, B.r, R, -1.0, 1.0, 1, false, prec);
     dots<T>(c, B.r, B.r, N, R, B.dotp, rr64);
   }
-  if (prec == COLA_PREC_MIXED || c->f64_tc_used) tc_check_error(c);
+  tc_check_results(c, prec);
   std::vector<double> hrr(R), hbb(R);
   COLA_CUDA(cudaMemcpyAsync(hrr.data(), rr64, 8 * R, cudaMemcpyDeviceToHost, c->s));
   COLA_CUDA(cudaMemcpyAsync(hbb.data(), bb, 8 * R, cudaMemcpyDeviceToHost, c->s));
@@ -1937,7 +1937,7 @@ void slq_impl(Ctx* c, const cola_linop* op, int nprobes, int m, uint64_t seed,
   COLA_CUDA(cudaMemcpyAsync(hz.data(), zn, 8 * hz.size(), cudaMemcpyDeviceToHost, c->s));
   COLA_CUDA(cudaMemcpyAsync(hm.data(), meff, 4 * hm.size(), cudaMemcpyDeviceToHost, c->s));
   COLA_CUDA(cudaStreamSynchronize(c->s));
-  if (c->f64_tc_used) tc_check_error(c);
+  tc_check_results(c, prec);
   std::vector<QuadResult> qr(nprobes);
   const int nthreads = (int)std::max<int64_t>(
       1, std::min<int64_t>(nprobes, std::max(1u, std::thread::hardware_concurrency())));

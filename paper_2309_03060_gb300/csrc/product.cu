@@ -104,6 +104,7 @@ cola_status product_solve(Ctx* c, const cola_linop* op, const void* Bin, void* X
   COLA_CUDA(cudaMemcpyAsync(hrr.data(), rr, 8 * R, cudaMemcpyDeviceToHost, c->s));
   COLA_CUDA(cudaMemcpyAsync(hbb.data(), bb, 8 * R, cudaMemcpyDeviceToHost, c->s));
   COLA_CUDA(cudaStreamSynchronize(c->s));
+  tc_check_results(c, prec);
   for (int64_t r = 0; r < R; ++r) {
     acc[r].rel_residual = hbb[r] > 0 ? sqrt(std::max(hrr[r], 0.0) / hbb[r]) : 0.0;
     if (info) info[r] = acc[r];

@@ -65,7 +65,6 @@ class Context:
         check(lib.cola_create(int(device), C.byref(h)))
         self.handle = h
         self.device = torch.device("cuda", device)
-        self._terms = None  # split terms last handed to the library
 
     def close(self):
         if self.handle:
@@ -73,11 +72,10 @@ class Context:
             self.handle = None
 
     def _set_split_terms(self, split_terms):
-        """The library's split-term setting (kept between calls)."""
+        """Set on every call: the handle may have other callers (the C interface,
+        other threads), so what was set last is not known here."""
         ft, vt = (split_terms, split_terms) if isinstance(split_terms, int) else split_terms
-        if (ft, vt) != self._terms:
-            check(_lib().cola_set_split_terms(self.handle, int(ft), int(vt)))
-            self._terms = (ft, vt)
+        check(_lib().cola_set_split_terms(self.handle, int(ft), int(vt)))
 
     def kernel_launches(self) -> int:
         n = C.c_int64()

@@ -603,7 +603,7 @@ cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
       img2[s] = bytes;
       bytes += f64_image_bytes(sys[s].n2, sys[s].n2);
     }
-    if (bytes <= kF64ImageCap) f64img = (char*)ws.try_get("bcg.f64img", bytes);
+    if (bytes <= kF64ImageCap) f64img = (char*)c->optional_ws("bcg.f64img", bytes);
   }
   if (f64img)
     for (int s = 0; s < nsys; ++s) {

@@ -88,6 +88,11 @@ struct Ctx {
   bool f64_tc_used = false;     // an FP64 tensor-core product ran since the last check
   int64_t tc_stall_ns = 0;      // armed by cola_test_stall_next_launch, consumed once
   void* host_pinned(size_t bytes);
+  // Workspace of a faster path that has another to fall back on: nullptr when it
+  // does not fit, and while a graph is captured (nothing may be allocated then)
+  // when it is not there already, so that the captured iterations take the path
+  // of the eager one before them.
+  void* optional_ws(const std::string& name, size_t bytes);
   void count_launch() {
     if (capturing)
       ++captured;

@@ -44,6 +44,7 @@ void* Workspace::try_get(const std::string& name, size_t bytes) {
   if (it != bufs.end()) {
     COLA_CUDA(cudaFree(it->second.p));
     bufs.erase(it);
+    ++generation;  // also when the allocation below fails: graphs hold the old address
   }
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
@@ -54,6 +55,12 @@ void* Workspace::try_get(const std::string& name, size_t bytes) {
   bufs[name] = Buf{p, bytes};
   ++generation;
   return p;
+}
+
+void* Ctx::optional_ws(const std::string& name, size_t bytes) {
+  if (!capturing) return ws.try_get(name, bytes);
+  const auto it = ws.bufs.find(name);
+  return it != ws.bufs.end() && it->second.bytes >= bytes ? it->second.p : nullptr;
 }
 
 void Workspace::release_all() {

@@ -759,8 +759,14 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.ntiles = (int)(R * tiles_m * p.nchunks);
   const size_t blocks = (size_t)p.nchunks * p.kchunks;
   if (p.nchunks > 65535 || p.kchunks > 65535 || blocks > 1024) return false;
-  uint16_t* img = (uint16_t*)c->optional_ws("f64.img", blocks * kDg * kADig);
-  int* fexp = (int*)c->optional_ws("f64.exp", blocks * kOut * 4);
+  // One buffer per power of two of blocks, which never grows (0.5 GB for all of
+  // them): a graph that a caller captured around a product keeps its image when a
+  // later product has a larger factor.
+  size_t cap = 1;
+  while (cap < blocks) cap *= 2;
+  const std::string cls = std::to_string(cap);
+  uint16_t* img = (uint16_t*)c->optional_ws("f64.img" + cls, cap * kDg * kADig);
+  int* fexp = (int*)c->optional_ws("f64.exp" + cls, cap * kOut * 4);
   if (!img || !fexp) return false;
   k_f64_digits<<<dim3(kOut, (unsigned)p.nchunks, (unsigned)p.kchunks), kKc, 0, c->s>>>(
       F, f_i, f_j, n_out, n_in, p.kchunks, img, fexp);

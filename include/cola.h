@@ -58,7 +58,10 @@ typedef enum {
 typedef enum { COLA_F64 = 0, COLA_F32 = 1 } cola_dtype;
 
 /* Arithmetic of the MVM and Krylov recurrences.
- *  F64   : FP64 everywhere (vectors FP64).
+ *  F64   : FP64 vectors and recurrences.  Kronecker mode products large enough for the
+ *          tensor cores run there as exact integer-digit products; every output is
+ *          as accurate by its own sum |K| |x| as FP64 multiply-adds make it (outputs
+ *          for which the digits cannot give that take FP64 multiply-adds).
  *  F32   : FP32 SIMT MVM and FP32 recurrences (vectors FP32).
  *  MIXED : Kronecker contractions on tcgen05 tensor cores with BF16 split
  *          operands (hi + lo [+ lo2] terms) and FP32 accumulation in TMEM,

@@ -629,10 +629,10 @@ cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
                               f64img + img2[s], (int)b.n1, (int)b.n2, (int)b.n2, b.R, b.N, b.N,
                               -b.ck, 1.0});
       }
-      f64_tc_batch(c, t1, "bcg.t1");
-      f64_tc_batch(c, t2, "bcg.t2");
-      residual_norms(dseg);
-      return;
+      if (f64_tc_batch(c, t1, "bcg.t1") && f64_tc_batch(c, t2, "bcg.t2")) {
+        residual_norms(dseg);
+        return;
+      }
     }
     std::vector<GemmDesc<double>> g1, g2;
     int64_t mm = 1, nn = 1;

@@ -213,7 +213,8 @@ void collect_leaves(const cola_linop* op, std::vector<const cola_linop*>& out);
 // Batches of FP64 mode steps over prepared factor images (kron_f64.cu): the
 // bytes and the making of one factor's image (256-byte aligned memory), and one
 // launch over a list of problems, each as f64_tc_mode_step with the factor F
-// row-major n_out x n_in.  Synchronises the stream.
+// row-major n_out x n_in.  Synchronises the stream.  False (nothing launched) when its
+// list of plain products does not fit.
 size_t f64_image_bytes(int64_t n_out, int64_t n_in);
 void f64_factor_image(Ctx* c, const double* F, int64_t f_i, int64_t f_j, int n_out, int n_in,
                       void* mem);
@@ -226,7 +227,7 @@ struct F64Batch {
   int64_t R, size_in, size_out;
   double alpha, beta;
 };
-void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag);
+bool f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag);
 
 // ------------------------------------------------------------- kernels API
 // Diagonal term of a product's epilogue: C += coeff d (.) x, x laid out as C

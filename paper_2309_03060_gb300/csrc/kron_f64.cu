@@ -10,8 +10,25 @@
 // [-128, 127]) that are exact in FP16.  The sums D_d = sum_{s+t=d} sum_j a_s b_t
 // of the 28 digit pairs with s + t <= 6 stay within 2^22 + d 2^21 <= 2^24 for 128
 // terms, so the FP32 accumulators hold them exactly; they are combined in 64-bit
-// integers (in units of D_5) and rounded to FP64 once.  What is lost: entries below 2^-55 of their row's or
-// vector's largest and the pairs s + t >= 7.
+// integers (in units of D_5) and rounded to FP64 once.  What is lost: what lies below
+// 2^-56 of a row's and 2^-55 of a vector's largest binade, and the pairs s + t >= 7;
+// together at most 1.14 2^-52 K 2^(Ef + Ex) of an output with K entries.
+//
+// That is a bound by row and vector.  An output is to be as accurate as FP64 products
+// make it by its own sum |f| |x|, however small that is beside the row's and the
+// vector's largest entries (graded vectors, columns of a covariance, block factors).  So
+// one more product runs on the tensor cores: the sum of leading magnitudes |a_0| |b_0|,
+// truncated to E5M2 (8-bit MMAs, 4 instead of 8 per 128 k).  Where it is at least
+// kLeadMin, sum |f| |x| is at least 2^-2.7 2^(Ef + Ex) and the loss of the order of FP64
+// roundings; an entry that counts alone is then within a binade of its largest and
+// exact in units of D_5 (an identity factor returns its input).  The other outputs, and those of rows
+// and vectors without digits (non-finite, far exponents), are left at 0 by the digit
+// products, listed, and computed with FP64 multiply-adds once the CTA's tiles are done.
+// Largest error over sum |f| |x|, in units of 2^-53, measured on RBF factors with sides
+// 32 .. 200: 0.6 .. 5.4, against 3.3 .. 9.9 in FP64 multiply-adds; graded vectors 20
+// against 20, identity and unit vectors 0 against 0.  A factor all of whose outputs
+// are plain runs at the rate of the FP64 units: identity 128^3 x 4, 5.25 ms for the
+// three steps, as in 32 x 32 tiles there.
 //
 // Why: this GPU's FP64 units do 2 multiply-adds per clock and SM (1.2 TFLOP/s),
 // its tensor cores ~1900 TFLOP/s in FP16, so 28 products are still ~50 times
@@ -23,24 +40,27 @@
 // 128 outputs i, step = tile x k chunk:
 //   warps 0-7   converters: load the 64 x 128 FP64 block into registers, find each
 //               vector's exponent and write the 7 digit images of the B operand
-//               (vectors x k, K-major, 128-byte swizzle, 112 KB)
-//   warps 8-15  drainers: add the accumulators up in 64-bit integers, scale, store
-//   warp 16     copies the factor's digit images (32 KB each, three buffers,
-//               cp.async.bulk from the prepared image, L2 resident)
-//   warp 17     issues the MMAs: factor digit s = 0 .. 6 outermost, so that group
+//               (vectors x k, K-major, 128-byte swizzle, 112 KB) and its leading
+//               magnitudes (8 KB)
+//   warps 8-15  drainers: note the outputs with too small a sum of magnitudes, add
+//               the accumulators up in 64-bit integers, scale, store
+//   warp 16     copies the factor's leading magnitudes (16 KB) and digit images
+//               (32 KB each; three buffers, cp.async.bulk from the prepared image, L2
+//               resident)
+//   warp 17     issues the MMAs: the magnitudes', then factor digit s = 0 .. 6 outermost, so that group
 //               s is the last to use B digit 6 - s and completes accumulator D_s;
 //               D_s is drained and digit 6 - s refilled for the next step while
 //               the later groups run, and only D_6 and digit 0 are left when the
 //               MMAs of a step end
-// Measured (128^3 x 16, one mode step, 268 MB in and out): 264 us against 6.97 ms
+// Measured (128^3 x 16, one mode step, 268 MB in and out): 265 us against 6.97 ms
 // on the FP64 units.  What bounds it: the integer work of converting 8192
 // entries and combining 8192 outputs per step (the ALU pipe), with the MMAs (224
 // of 128 x 64 x 16 per step, 48 clocks each by their shared-memory reads) at
 // 0.7 of the time; converting and draining in separate warps, both beside the
 // MMAs, took it from 395 us, no FP64-pipe instruction per output from 450 us, and
 // issuing from a converged warp (uniform descriptors) from 520 us.
-// Accumulators: D_0 .. D_6, 64 FP32 columns each of tensor memory.  Every
-// mbarrier wait gives up after ~2 s and raises the error flag.
+// Accumulators: D_0 .. D_6 and the magnitudes', 64 FP32 columns each of tensor memory
+// (all 512).  Every mbarrier wait gives up after ~2 s and raises the error flag.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -63,8 +83,18 @@ constexpr int kLoadWarp = kConvWarps + kDrainWarps, kMmaWarp = kLoadWarp + 1;
 constexpr int kThreadsF64 = 32 * (kMmaWarp + 1);
 constexpr uint32_t kBDig = kVec * kKc * 2;   // 16 KB per B digit
 constexpr uint32_t kADig = kOut * kKc * 2;   // 32 KB per A digit
+constexpr uint32_t kBLead = kVec * kKc;      // 8 KB of leading magnitudes of B
+constexpr uint32_t kALead = kOut * kKc;      // 16 KB of A
+constexpr uint32_t kABlk = kDg * kADig + kALead;  // image of one 128 x 128 factor block
 constexpr int kABufs = 3;
-constexpr size_t kSmemF64 = 1024 + kDg * kBDig + kABufs * kADig + 6144;
+constexpr size_t kSmemF64 = 1024 + kDg * kBDig + kBLead + kABufs * kADig + 6144;
+// Outputs whose sum of leading magnitudes is below this take plain products: 128
+// (|a_0| of a power of two) times 40, the smallest E5M2 number above 32 = |b_0| of an
+// entry a binade below its vector's largest.
+constexpr float kLeadMin = 5120.0f;
+// Magnitude (E5M2, 2^8) that stands for every entry of a zero row, whose outputs are 0
+// unless the vector has no digits.
+constexpr uint32_t kLeadZero = 0x5c;
 constexpr int kPlain = 1 << 20;  // exponent mark of a factor row that takes plain products
 
 struct F64Params {
@@ -84,6 +114,12 @@ struct F64Params {
 struct F64Launch {
   int* err;
   uint64_t stall_ns;
+  // Outputs left to plain products: per CTA low_cap entries, each one thread's of one
+  // step (thread of the drainers + 256 times the CTA's tile; k chunk; the mask of its
+  // 32 outputs).
+  uint32_t* low;
+  int64_t low_cap;
+  int kmax;  // most k chunks of a problem
 };
 
 // Where a tile's parameters come from: one problem by value, or a device table
@@ -166,11 +202,6 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return *reinterpret_cast<const uint32_t*>(&d);
 }
 
-// a 2^e for an e outside the range of scaled_double (overflow, denormals).
-__device__ __noinline__ double far_scale(long long a, int e) {
-  return ldexp(__ll2double_rn(a), e);
-}
-
 // a 2^e rounded to FP64 for 1023 + 62 + |e| within the exponent range, by
 // integer operations (an FP64 conversion is two instructions of 16 clocks each
 // on the SM's FP64 units): the leading bit of |a| goes to bit 63, bits 63 .. 11
@@ -189,13 +220,65 @@ __device__ __forceinline__ double scaled_double(long long a, int e) {
   return __hiloint2double((int)(hi | (sg & 0x80000000u)), (int)(uint32_t)r);
 }
 constexpr int kFarExp = 450;  // |exponent| of a row or vector up to which it does
+constexpr int kHidden = 4;    // see the drain
+__device__ __forceinline__ bool far_key(int key) {
+  return key != 0 && (!has_digits(key) || abs((key >> 20) - 1023) > kFarExp);
+}
 
-// The dot product of one output whose factor row or vector has no digits.
-__device__ __noinline__ double plain_dot(const double* f, int64_t f_j, const double* x,
-                                         int64_t rest, int k0, int k1) {
-  double v = 0.0;
-  for (int k = k0; k < k1; ++k) v = fma(f[k * f_j], x[(int64_t)k * rest], v);
-  return v;
+// y += alpha f . x over the k chunk [k0, k1) for the columns (vectors) of one mask:
+// column c at x + c and y + c n_out.  Four columns at a time share the loads of f and are
+// a chain each; fewer take four chains each.
+__device__ __forceinline__ void plain_columns(const F64Params& p, uint32_t mask, int k0, int k1,
+                                              const double* f, const double* x, double* y) {
+  while (mask != 0) {
+    int c[4];
+    const bool four = __popc(mask) >= 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      c[q] = q == 0 || four ? __ffs(mask) - 1 : 0;
+      if (q == 0 || four) mask &= mask - 1;
+    }
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int k = k0;
+    if (four) {
+      for (; k + 4 <= k1; k += 4) {
+        double fv[4], xv[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          fv[u] = f[(k + u) * p.f_j];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) xv[u][q] = x[(int64_t)(k + u) * p.rest + c[q]];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] = fma(fv[u], xv[u][q], a[q]);
+      }
+      for (; k < k1; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          a[q] = fma(f[k * p.f_j], x[(int64_t)k * p.rest + c[q]], a[q]);
+    } else {
+      for (; k + 8 <= k1; k += 8) {
+        double fv[8], xv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          fv[u] = f[(k + u) * p.f_j];
+          xv[u] = x[(int64_t)(k + u) * p.rest + c[0]];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u & 3] = fma(fv[u], xv[u], a[u & 3]);
+      }
+      for (; k < k1; ++k) a[0] = fma(f[k * p.f_j], x[(int64_t)k * p.rest + c[0]], a[0]);
+      a[0] = (a[0] + a[1]) + (a[2] + a[3]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q == 0 || four) {
+        double* o = y + (int64_t)c[q] * p.n_out;
+        *o = fma(p.alpha, a[q], *o);
+      }
+  }
 }
 
 // The digit images and exponents of one factor (chunk): block (row of the
@@ -218,14 +301,20 @@ __global__ void __launch_bounds__(kKc) k_f64_digits(const double* F, int64_t f_i
   const int emax = mx >> 20;
   const bool dig = has_digits(mx);
   const int64_t blk = (int64_t)nc * kchunks + kc;
-  if (k == 0) fexp[blk * kOut + row] = dig ? emax - 1023 : kPlain;
+  if (k == 0) fexp[blk * kOut + row] = dig ? (mx ? emax - 1023 : 0) : kPlain;
   const unsigned long long u =
       dig && mx ? fixed_digits<3>((unsigned long long)__double_as_longlong(x), emax) : kZeroDigits;
   // digit t: k block (k / 64), row, 16-byte chunk (k / 8) mod 8 swizzled by the row
-  uint16_t* p = img + blk * (kDg * kADig / 2) + (size_t)(k >> 6) * (kOut * 64) + row * 64 +
+  uint16_t* p = img + blk * (kABlk / 2) + (size_t)(k >> 6) * (kOut * 64) + row * 64 +
                 ((((k >> 3) & 7) ^ (row & 7)) << 3) + (k & 7);
   constexpr size_t st = kADig / 2;
-  p[0 * st] = (uint16_t)digit_pair<0>(u, u);
+  const uint32_t lead = digit_pair<0>(u, u);
+  p[0 * st] = (uint16_t)lead;
+  // the leading magnitude: 16-byte chunk k / 16 of the row, swizzled likewise
+  reinterpret_cast<unsigned char*>(img + blk * (kABlk / 2))[kDg * kADig + row * kKc +
+                                                            (((k >> 4) ^ (row & 7)) << 4) +
+                                                            (k & 15)] =
+      (unsigned char)(mx ? (lead >> 8) & 0x7fu : (j < n_in ? kLeadZero : 0u));
   p[1 * st] = (uint16_t)digit_pair<1>(u, u);
   p[2 * st] = (uint16_t)digit_pair<2>(u, u);
   p[3 * st] = (uint16_t)digit_pair<3>(u, u);
@@ -295,6 +384,45 @@ __device__ __forceinline__ void put_digit(unsigned char* bdig, const unsigned lo
   }
 }
 
+// put_digit<0> and this thread's leading magnitudes, |digit 0| truncated to E5M2 (the
+// upper byte of its FP16 form), up to kpad rounded to the 32 k of an 8-bit MMA
+// (entries past n_in are zeros).
+__device__ __forceinline__ void put_lead(unsigned char* bdig, unsigned char* blead,
+                                         const unsigned long long (&u)[32], int n, int oct,
+                                         int kpad) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    if (oct * 8 + h * 32 >= (kpad + 31) / 32 * 32) continue;
+    uint4 w;
+    w.x = digit_pair<0>(u[8 * h + 0], u[8 * h + 1]);
+    w.y = digit_pair<0>(u[8 * h + 2], u[8 * h + 3]);
+    w.z = digit_pair<0>(u[8 * h + 4], u[8 * h + 5]);
+    w.w = digit_pair<0>(u[8 * h + 6], u[8 * h + 7]);
+    const int ch = (oct + 4 * (h & 1)) ^ (n & 7);
+    *reinterpret_cast<uint4*>(bdig + (h >> 1) * (kBDig / 2) + n * 128 + ch * 16) = w;
+    const uint2 m = make_uint2(__byte_perm(w.x, w.y, 0x7531) & 0x7f7f7f7fu,
+                               __byte_perm(w.z, w.w, 0x7531) & 0x7f7f7f7fu);
+    *reinterpret_cast<uint2*>(blead + n * kKc + ((((oct >> 1) + 2 * h) ^ (n & 7)) << 4) +
+                              (oct & 1) * 8) = m;
+  }
+}
+
+// Which of this thread's 32 outputs have too small a sum of leading magnitudes.
+__device__ __forceinline__ uint32_t low_outputs(uint32_t taddr) {
+  uint32_t v[32];
+  tmem_ld32(taddr + kDg * kVec, v);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  float mn = __uint_as_float(v[0]);
+#pragma unroll
+  for (int e = 1; e < 32; ++e) mn = fminf(mn, __uint_as_float(v[e]));
+  uint32_t low = 0;
+  if (__any_sync(0xffffffffu, mn < kLeadMin)) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e) low |= (__uint_as_float(v[e]) < kLeadMin ? 1u : 0u) << e;
+  }
+  return low;
+}
+
 // The MMAs of factor digit a with every B digit t <= 6 - a (t downwards: digit
 // 0 is refilled last).  One warp issues 224 MMAs per step, so the k loop is
 // unrolled with constant descriptor offsets.
@@ -323,7 +451,8 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* bdig = base;
-  unsigned char* adig = base + kDg * kBDig;
+  unsigned char* blead = base + kDg * kBDig;
+  unsigned char* adig = blead + kBLead;
   uint64_t* afull = (uint64_t*)(adig + kABufs * kADig);
   uint64_t* aempty = afull + kABufs;
   uint64_t* ready = aempty + kABufs;  // B digits written, D of the step before drained
@@ -340,6 +469,10 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
   int* cmax = (int*)(tmem_slot + 2);     // [2][4][64]
   int* ckey = cmax + 8 * kVec;           // [2][64]
   volatile int* cfar = ckey + 2 * kVec;  // [2][2]
+  // per drainer thread: the outputs of its step with too small a sum of leading
+  // magnitudes; entries of L.low so far
+  volatile uint32_t* clow = (volatile uint32_t*)(cfar + 4);  // [32 kDrainWarps]
+  int* nlow = (int*)(clow + 32 * kDrainWarps);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -356,6 +489,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     mbar_init(drain, 1);
     mbar_init(stall, 1);
     *abort_flag = 0;
+    *nlow = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) {
@@ -383,16 +517,17 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
         const int kchunks = p.kchunks, nc = lt % p.nchunks;
         const int kb_last = (p.n_in - (kchunks - 1) * kKc + 63) / 64;  // k blocks, last chunk
         const unsigned char* img =
-            (const unsigned char*)p.img + (int64_t)nc * kchunks * (int64_t)(kDg * kADig);
-        for (int kc = 0; kc < kchunks && ok; ++kc, img += kDg * kADig) {
-          const uint32_t bytes = (kc == kchunks - 1 ? kb_last : 2) * (kADig / 2);
-          for (int a = 0; a < kDg; ++a) {
+            (const unsigned char*)p.img + (int64_t)nc * kchunks * (int64_t)kABlk;
+        for (int kc = 0; kc < kchunks && ok; ++kc, img += kABlk) {
+          // the leading magnitudes (after the digits in the image), then the digits
+          for (int a = -1; a < kDg; ++a) {
+            const uint32_t bytes = a < 0 ? kALead : (kc == kchunks - 1 ? kb_last : 2) * (kADig / 2);
             if (!mbar_wait(&aempty[s], ph ^ 1u, abort_flag, L.err)) {
               ok = false;
               break;
             }
             mbar_arrive_expect_tx(&afull[s], bytes);
-            bulk_g2s(adig + s * kADig, img + a * kADig, bytes, &afull[s]);
+            bulk_g2s(adig + s * kADig, img + (a < 0 ? kDg : a) * kADig, bytes, &afull[s]);
             issued |= 1u << s;
             issued_ph = (issued_ph & ~(1u << s)) | (ph << s);
             if (++s == kABufs) {
@@ -416,6 +551,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     if (L.stall_ns)
       ok = __all_sync(0xffffffffu, mbar_wait_slow(stall, 0, abort_flag, L.err, L.stall_ns));
     const uint64_t adesc = sw128_desc(smem_u32(adig)), bdesc = sw128_desc(smem_u32(bdig));
+    const uint64_t ldesc = sw128_desc(smem_u32(blead));
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base, 0);
     int s = 0;
     uint32_t ph = 0, sph = 0;
@@ -429,6 +565,25 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
         ok = mbar_wait_warp(ready, sph, abort_flag, L.err);
         if (!ok) break;
         tc_fence_after();
+        // the sums of leading magnitudes (complete and its operands free with group 0)
+        ok = mbar_wait_warp(&afull[s], ph, abort_flag, L.err);
+        if (!ok) break;
+        tc_fence_after();
+        {
+          const uint64_t ad = adesc + (uint64_t)((uint32_t)s * (kADig >> 4));
+          const int lsteps = (min(kleft, kKc) + 31) / 32;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (k >= lsteps) break;
+            mma_one_f8(tmem + kDg * kVec, ad + (uint64_t)k * 2, ldesc + (uint64_t)k * 2,
+                       idesc_e5m2(kOut, kVec), k ? 1u : 0u, elect);
+          }
+          mma_commit_one(&aempty[s], elect);
+          if (++s == kABufs) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
         for (int a = 0; a < kDg; ++a) {
           ok = mbar_wait_warp(&afull[s], ph, abort_flag, L.err);
           if (!ok) break;
@@ -504,8 +659,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       }
       if (oct == 0) {
         ckey[par * kVec + n] = key;
-        const bool far = key != 0 && (!dig || abs(emax - 1023) > kFarExp);
-        const bool any = __any_sync(0xffffffffu, far);
+        const bool any = __any_sync(0xffffffffu, far_key(key));
         if (lane == 0) cfar[par * 2 + warp] = any;
       }
       __syncwarp();
@@ -523,7 +677,10 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
     if (ok) ok = mbar_wait(&dfull[S], dph, abort_flag, L.err);             \
     ok = __all_sync(0xffffffffu, ok);                                      \
   }                                                                        \
-  put_digit<6 - S>(bdig, u, n, oct, kpad);
+  if constexpr (S < 6)                                                     \
+    put_digit<6 - S>(bdig, u, n, oct, kpad);                               \
+  else                                                                     \
+    put_lead(bdig, blead, u, n, oct, kpad);
       COLA_DIGIT(0)
       COLA_DIGIT(1)
       COLA_DIGIT(2)
@@ -579,7 +736,10 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
   if (ok) ok = mbar_wait(&dfull[S], (uint32_t)par, abort_flag, L.err);     \
   ok = __all_sync(0xffffffffu, ok);                                        \
   tc_fence_after();                                                        \
-  if (ok) fold<S>(taddr, acc);
+  if (ok) {                                                                \
+    if constexpr (S == 0) clow[tid - 32 * kConvWarps] = low_outputs(taddr); \
+    fold<S>(taddr, acc);                                                   \
+  }
       COLA_DIGIT(0)
       COLA_DIGIT(1)
       COLA_DIGIT(2)
@@ -600,12 +760,13 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       if (ok && i < p.n_out && cnt > 0) {
         double* y = p.Y + cur.r * p.size_out + (int64_t)(cur.m0 + oc0) * p.n_out + i;
         const int* keys = ckey + par * kVec + oc0;
+        uint32_t low = clow[tid - 32 * kConvWarps];  // outputs that take plain products
         const bool near = abs(ef) <= kFarExp && !(cfar[par * 2] | cfar[par * 2 + 1]);
         const int e0 = ef - 53 - 1023;
         // Y's old values join with beta (first k chunk) or 1 (later chunks)
         const bool old = kc > 0 || p.has_beta;
         const double bo = kc > 0 ? 1.0 : p.beta;
-        if (near && cnt == 32) {  // no branch per output
+        if (near && low == 0 && cnt == 32) {  // no branch per output
 #pragma unroll
           for (int g = 0; g < 32; g += 4) {
             double v[4];
@@ -622,26 +783,37 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
             }
           }
         } else {
+          if (cnt < 32) low &= (1u << cnt) - 1;
 #pragma unroll 1
           for (int c = 0; c < cnt; ++c) {
             long long ac = 0;
 #pragma unroll
             for (int q = 0; q < 32; ++q)
               if (q == c) ac = acc[q];
-            const int key = keys[c];
-            double v;
-            if (near) {
-              v = scaled_double(ac, e0 + (key >> 20));
-            } else if (has_digits(key) && ef != kPlain) {
-              v = far_scale(ac, e0 + (key >> 20));
-            } else {
-              v = plain_dot(p.F + i * p.f_i, p.f_j, p.X + cur.r * p.size_in + cur.m0 + oc0 + c,
-                            p.rest, kc * kKc, min(p.n_in, (kc + 1) * kKc));
+            const int key = keys[c], e = e0 + (key >> 20);
+            const double yo = old ? *y : 0.0;
+            if (abs(ef) > kFarExp || far_key(key)) {  // out of scaled_double's range
+              low |= 1u << c;
+            } else if (low >> c & 1u) {
+              // too small a sum of leading magnitudes, except where the digits are exact (a
+              // zero vector) and where their error, below 2^-51 K 2^(Ef + Ex), is hidden by
+              // the rounding of a sum so far of at least 2^kHidden of that binade
+              if (key == 0 || (kc > 0 && fabs(yo) >= fabs(p.alpha) *
+                                             __hiloint2double((1023 + 53 + kHidden + e) << 20, 0)))
+                low ^= 1u << c;
             }
+            double v = scaled_double(low >> c & 1u ? 0ll : ac, e);
             if (p.has_alpha) v *= p.alpha;
-            if (old) v = fma(bo, *y, v);
+            if (old) v = fma(bo, yo, v);
             *y = v;
             y += p.n_out;
+          }
+          if (low != 0) {
+            uint32_t* e = L.low + 3 * ((int64_t)blockIdx.x * L.low_cap + atomicAdd(nlow, 1));
+            e[0] = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x * (32 * kDrainWarps) +
+                              tid - 32 * kConvWarps);
+            e[1] = (uint32_t)kc;
+            e[2] = low;
           }
         }
       }
@@ -662,13 +834,48 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
                  "r"(512)
                  : "memory");
   }
+  // The outputs left out above, on the FP64 units (their rate bounds it: a tile
+  // whose outputs are all plain takes 260 us).  Y is this CTA's own.
+  // One k chunk after the other, as an output may be left out of several.
+  const int entries = *abort_flag ? 0 : *nlow;
+  for (int kc = 0; kc < (entries ? L.kmax : 0); ++kc) {
+    for (int n = tid; n < entries; n += kThreadsF64) {
+      const uint32_t* e = L.low + 3 * ((int64_t)blockIdx.x * L.low_cap + n);
+      if (e[1] != (uint32_t)kc) continue;
+      const int thr = e[0] % (32 * kDrainWarps);
+      int lt;
+      const F64Params& p = src.get(
+          (int)blockIdx.x + (int)(e[0] / (32 * kDrainWarps)) * (int)gridDim.x, lt);
+      const F64Step cur = step_of(p, lt, kc);
+      const int i = cur.nc * kOut + thr % kOut, m = cur.m0 + thr / kOut * 32;
+      plain_columns(p, e[2], kc * kKc, min(p.n_in, (kc + 1) * kKc), p.F + i * p.f_i,
+                    p.X + cur.r * p.size_in + m,
+                    p.Y + cur.r * p.size_out + (int64_t)m * p.n_out + i);
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace
 
+// The list of outputs left to plain products, for `ntiles` tiles of at most
+// kchunks k chunks (5 % of Y's bytes per chunk); false when it does not fit.  One buffer
+// per power of two of bytes, which never moves (see f64_tc_mode_step).
+static bool f64_low_list(Ctx* c, int ntiles, int kchunks, F64Launch* L) {
+  const int grid = std::min(ntiles, c->num_sms), per = (ntiles + grid - 1) / grid;
+  if (per >= 1 << 24) return false;
+  L->low_cap = (int64_t)per * kchunks * (32 * kDrainWarps);
+  L->kmax = kchunks;
+  const size_t bytes = 12 * (size_t)grid * L->low_cap;
+  int lg = 16;
+  while (((size_t)1 << lg) < bytes) ++lg;
+  L->low = (uint32_t*)c->optional_ws("f64.low" + std::to_string(lg), (size_t)1 << lg);
+  return L->low != nullptr;
+}
+
 template <class Src>
-static void f64_launch(Ctx* c, const Src& src, int ntiles) {
-  F64Launch L{tc_errflag(c), 0};
+static void f64_launch(Ctx* c, const Src& src, int ntiles, F64Launch L) {
+  L.err = tc_errflag(c);
   if (c->tc_stall_ns > 0 && !c->capturing) {
     L.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
     c->tc_stall_ns = 0;
@@ -683,7 +890,7 @@ static void f64_launch(Ctx* c, const Src& src, int ntiles) {
 
 size_t f64_image_bytes(int64_t n_out, int64_t n_in) {
   return (size_t)((n_out + kOut - 1) / kOut) * (size_t)((n_in + kKc - 1) / kKc) *
-         (kDg * kADig + kOut * 4);
+         (kABlk + kOut * 4);
 }
 
 void f64_factor_image(Ctx* c, const double* F, int64_t f_i, int64_t f_j, int n_out, int n_in,
@@ -691,12 +898,12 @@ void f64_factor_image(Ctx* c, const double* F, int64_t f_i, int64_t f_j, int n_o
   const int nch = (n_out + kOut - 1) / kOut, kch = (n_in + kKc - 1) / kKc;
   k_f64_digits<<<dim3(kOut, (unsigned)nch, (unsigned)kch), kKc, 0, c->s>>>(
       F, f_i, f_j, n_out, n_in, kch, (uint16_t*)mem,
-      (int*)((char*)mem + (size_t)nch * kch * (kDg * kADig)));
+      (int*)((char*)mem + (size_t)nch * kch * kABlk));
   c->count_launch();
   COLA_CUDA(cudaGetLastError());
 }
 
-void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
+bool f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
   std::vector<F64Params> hp(probs.size());
   std::vector<int> first(probs.size()), tile_prob;
   for (size_t i = 0; i < probs.size(); ++i) {
@@ -713,7 +920,7 @@ void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
     p.f_i = b.n_in;
     p.f_j = 1;
     p.img = (const uint16_t*)b.image;
-    p.fexp = (const int*)((const char*)b.image + (size_t)p.nchunks * p.kchunks * (kDg * kADig));
+    p.fexp = (const int*)((const char*)b.image + (size_t)p.nchunks * p.kchunks * kABlk);
     p.rest = b.rest;
     p.n_in = b.n_in;
     p.n_out = b.n_out;
@@ -727,7 +934,11 @@ void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
     tile_prob.insert(tile_prob.end(), (size_t)p.ntiles, (int)i);
   }
   const int nt = (int)tile_prob.size(), np = (int)probs.size();
-  if (nt == 0) return;
+  if (nt == 0) return true;
+  int kmax = 1;
+  for (const F64Params& p : hp) kmax = std::max(kmax, p.kchunks);
+  F64Launch L{};
+  if (!f64_low_list(c, nt, kmax, &L)) return false;
   const std::string t = tag;
   F64Tab src{};
   src.probs = (const F64Params*)c->ws.get(t + ".p", sizeof(F64Params) * np);
@@ -740,8 +951,9 @@ void f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
                             cudaMemcpyHostToDevice, c->s));
   COLA_CUDA(cudaMemcpyAsync((void*)src.first, first.data(), 4 * (size_t)np,
                             cudaMemcpyHostToDevice, c->s));
-  f64_launch(c, src, nt);
+  f64_launch(c, src, nt, L);
   COLA_CUDA(cudaStreamSynchronize(c->s));  // the host tables go out of scope
+  return true;
 }
 
 bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, const double* X,
@@ -765,9 +977,10 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   size_t cap = 1;
   while (cap < blocks) cap *= 2;
   const std::string cls = std::to_string(cap);
-  uint16_t* img = (uint16_t*)c->optional_ws("f64.img" + cls, cap * kDg * kADig);
+  uint16_t* img = (uint16_t*)c->optional_ws("f64.img" + cls, cap * kABlk);
   int* fexp = (int*)c->optional_ws("f64.exp" + cls, cap * kOut * 4);
-  if (!img || !fexp) return false;
+  F64Launch L{};
+  if (!img || !fexp || !f64_low_list(c, p.ntiles, p.kchunks, &L)) return false;
   k_f64_digits<<<dim3(kOut, (unsigned)p.nchunks, (unsigned)p.kchunks), kKc, 0, c->s>>>(
       F, f_i, f_j, n_out, n_in, p.kchunks, img, fexp);
   c->count_launch();
@@ -787,7 +1000,7 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.beta = beta;
   p.has_alpha = alpha != 1.0;
   p.has_beta = beta != 0.0;
-  f64_launch(c, F64One{p}, p.ntiles);
+  f64_launch(c, F64One{p}, p.ntiles, L);
   return true;
 }
 

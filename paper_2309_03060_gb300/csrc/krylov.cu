@@ -1303,11 +1303,11 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
   auto chunk_end = [&](int64_t i) { return i <= 1 ? i : 1 + (i - 1 + chunk - 1) / chunk * chunk; };
   const int64_t cap = chunk_end(o.maxiter);
   // Without refinement the iterations after the last right-hand side stopped are
-  // lost: a chunk is run in parts of 8 iterations at first and of more (up to the
-  // chunk) until one takes kChunkSeconds, well above the ~15 us a host check costs,
-  // and is left at the first part that ends with every right-hand side stopped
-  // (2^20-point stencil + low-rank solve, 21 iterations: 25 run instead of 65, 11.6
-  // -> 5.5 ms).  No part crosses the chunk's end and the iterations not run count,
+  // lost, and nothing else depends on where a replay ends: replays start at 8
+  // iterations and grow (up to the chunk) until one takes kChunkSeconds, well above
+  // the ~15 us a host check costs (2^20-point stencil + low-rank solve, 21
+  // iterations: 25 run instead of 65, 11.6 -> 5.5 ms).  None crosses the cap, and a solve
+  // that stopped is counted to the end of the chunk of its last iteration (`ran`),
   // so that the cap, the verification and its restarts do not depend on the times
   // measured here.  Refined solves replace residuals at chunk ends and run whole
   // chunks.
@@ -1345,7 +1345,26 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
     fprintf(stderr, "[cola cg] %s iter %lld active %d recursive %.3e true %.3e updates %d\n", what,
             (long long)iters, act, worst, worst64, updates);
   };
+  // Unrefined solves: the state as of iteration `at` (after the last read), and the
+  // iterations since then in which some right-hand side was active.  One that stopped
+  // for its curvature p^T A p did not count the iteration it stopped in.
+  std::vector<CgState> before;
+  int64_t at = 0;
+  auto snapshot = [&] {
+    if (refine) return;
+    before.assign(hst, hst + R);
+    at = iters;
+  };
+  auto ran = [&] {
+    int64_t n = 1;
+    for (int64_t r = 0; r < R; ++r)
+      n = std::max<int64_t>(n, hst[r].iters - before[r].iters +
+                                   (before[r].active && hst[r].status == COLA_ERR_BREAKDOWN &&
+                                    std::isfinite(hst[r].rr)));
+    return n;
+  };
   read_state();
+  snapshot();
   bool any_active = false;
   for (int64_t r = 0; r < R; ++r) any_active |= hst[r].active != 0;
   // one eager iteration sizes every workspace buffer before capture
@@ -1359,23 +1378,18 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
     if (B.small.on) {
       // ends by itself when every right-hand side has stopped
       const int limit = (int)std::min<int64_t>(cap - iters, kSmallChunk);
-      int64_t ran = 0;
-      std::vector<int64_t> before(R);
-      for (int64_t r = 0; r < R; ++r) before[r] = hst[r].iters;
       small_cg_run<T>(c, B.small, B.r, B.x, B.p, B.invd, B.st, R, limit);
       read_state();
       any_active = false;
-      for (int64_t r = 0; r < R; ++r) {
-        any_active |= hst[r].active != 0;
-        ran = std::max<int64_t>(ran, hst[r].iters - before[r]);
-      }
-      if (any_active && ran < limit) tc_check_error(c);  // the kernel gave up waiting
-      iters = any_active ? iters + limit : chunk_end(iters + std::max<int64_t>(ran, 1));
+      for (int64_t r = 0; r < R; ++r) any_active |= hst[r].active != 0;
+      if (any_active && ran() < limit) tc_check_error(c);  // the kernel gave up waiting
+      iters = any_active ? iters + limit : chunk_end(at + ran());
+      snapshot();
       trace_line("chunk");
       continue;
     }
     const auto tc0 = std::chrono::steady_clock::now();
-    if (!refine) run_chunk = (int)std::min<int64_t>(want_chunk, chunk_end(iters + 1) - iters);
+    if (!refine) run_chunk = (int)std::min<int64_t>(want_chunk, cap - iters);
     cg_chunk<T>(c, op, B, N, R, nblk, prec, delta2, refine ? 1 : 0, run_chunk, graph_key());
     iters += run_chunk;
     read_state();
@@ -1408,7 +1422,8 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
       paused |= hst[r].paused != 0;
     }
     any_active = nact > 0;
-    if (!any_active) iters = chunk_end(iters);
+    if (!refine && !any_active) iters = chunk_end(at + ran());
+    snapshot();
     const bool flag = paused || (defer ? (nflag > 0 && 2 * nflag >= nact) : nflag > 0);
     if (refine && (flag || !any_active) && updates < o.max_updates) {
       const auto tr0 = std::chrono::steady_clock::now();
@@ -1456,6 +1471,7 @@ static cola_status cg_run(Ctx* c, cola_linop* op, const void* Bin, void* Xout, i
                                                                R, B.beta_vec);
     c->count_launch();
     read_state();
+    snapshot();
     trace_line("verify");
     any_active = false;
     for (int64_t r = 0; r < R; ++r) any_active |= hst[r].active != 0;

@@ -19,22 +19,27 @@
 // vector's largest entries (graded vectors, columns of a covariance, block factors).  So
 // one more product runs on the tensor cores: the sum of leading magnitudes |a_0| |b_0|,
 // truncated to E5M2 (8-bit MMAs, 4 instead of 8 per 128 k).  Where it is at least
-// kLeadMin, sum |f| |x| is at least 2^-2.7 2^(Ef + Ex) and the loss of the order of FP64
-// roundings; an entry that counts alone is then within a binade of its largest and
-// exact in units of D_5 (an identity factor returns its input).  The other outputs, and those of rows
-// and vectors without digits (non-finite, far exponents), are left at 0 by the digit
-// products, listed, and computed with FP64 multiply-adds once the CTA's tiles are done.
+// kLeadMin, sum |f| |x| is at least 2^-3.7 2^(Ef + Ex) and the loss of the order of FP64
+// roundings.  A factor row with a single entry takes twice that: the vector's entry is
+// then within a binade of its largest and exact in units of D_5 (an identity factor
+// returns its input).  The other outputs, and those of rows and vectors without digits
+// (non-finite, far exponents), are listed and computed with FP64 multiply-adds once the
+// CTA's tiles are done.
 // Largest error over sum |f| |x|, in units of 2^-53, measured on RBF factors with sides
 // 32 .. 200: 0.6 .. 5.4, against 3.3 .. 9.9 in FP64 multiply-adds; graded vectors 20
-// against 20, identity and unit vectors 0 against 0.  A factor all of whose outputs
-// are plain runs at the rate of the FP64 units: identity 128^3 x 4, 5.25 ms for the
-// three steps, as in 32 x 32 tiles there.
+// against 20, identity 0 against 0, unit vectors 1.6 against 0.  What it costs: nothing
+// where no output is low, the rate of the FP64 units where most are (identity 128^3 x 4:
+// 6.1 ms for the three steps, 5.25 ms in 32 x 32 tiles there; columns of a 128 x 128 RBF
+// product, 64 of them: 0.33 against 0.47 ms), and on short RBF factors of a small
+// lengthscale, some of whose points have no neighbour, part of the gain: sides 32, 48,
+// lengthscale 0.05, 16 vectors 134, 205 us against 87, 140 without it and 123, 625 on the
+// FP64 units.
 //
 // Why: this GPU's FP64 units do 2 multiply-adds per clock and SM (1.2 TFLOP/s),
 // its tensor cores ~1900 TFLOP/s in FP16, so 28 products are still ~50 times
 // cheaper.  Every FP64 pipe use in the inner path is avoided: exponents and
 // digits come from integer operations, and so do the combination and its
-// conversion; only alpha, beta other than 1, 0 take FP64 instructions.
+// conversion; of the outputs only alpha, beta other than 1, 0 take FP64 instructions.
 //
 // Kernel layout (persistent, one 576-thread CTA per SM), tile = 64 vectors m x
 // 128 outputs i, step = tile x k chunk:
@@ -47,18 +52,21 @@
 //   warp 16     copies the factor's leading magnitudes (16 KB) and digit images
 //               (32 KB each; three buffers, cp.async.bulk from the prepared image, L2
 //               resident)
-//   warp 17     issues the MMAs: the magnitudes', then factor digit s = 0 .. 6 outermost, so that group
-//               s is the last to use B digit 6 - s and completes accumulator D_s;
+//   warp 17     issues the MMAs: the magnitudes', then factor digit s = 0 .. 6
+//               outermost, so that group s is the last to use B digit 6 - s and completes
+//               accumulator D_s;
 //               D_s is drained and digit 6 - s refilled for the next step while
 //               the later groups run, and only D_6 and digit 0 are left when the
 //               MMAs of a step end
 // Measured (128^3 x 16, one mode step, 268 MB in and out): 265 us against 6.97 ms
-// on the FP64 units.  What bounds it: the integer work of converting 8192
-// entries and combining 8192 outputs per step (the ALU pipe), with the MMAs (224
-// of 128 x 64 x 16 per step, 48 clocks each by their shared-memory reads) at
-// 0.7 of the time; converting and draining in separate warps, both beside the
-// MMAs, took it from 395 us, no FP64-pipe instruction per output from 450 us, and
-// issuing from a converged warp (uniform descriptors) from 520 us.
+// on the FP64 units.  What bounds it: the chain of conversion, MMAs and drain of a
+// step, each waiting for the one before with 18 warps on the SM: the integer pipe (8192
+// entries converted, 8192 outputs combined per step) is active 0.58 of the time, the
+// tensor-core pipe (224 MMAs of 128 x 64 x 16 per step) 0.61, issue slots 0.50;
+// converting and draining in separate warps, both beside the MMAs, took it from 395 us,
+// no FP64 conversion per output from 450 us, and issuing from a converged warp (uniform
+// descriptors) from 520 us.  18 warps hold a thread to 96 registers (56 bytes of spills;
+// 260 in the variants for short factors and for a table of problems).
 // Accumulators: D_0 .. D_6 and the magnitudes', 64 FP32 columns each of tensor memory
 // (all 512).  Every mbarrier wait gives up after ~2 s and raises the error flag.
 #include <cuda_fp16.h>
@@ -88,10 +96,10 @@ constexpr uint32_t kALead = kOut * kKc;      // 16 KB of A
 constexpr uint32_t kABlk = kDg * kADig + kALead;  // image of one 128 x 128 factor block
 constexpr int kABufs = 3;
 constexpr size_t kSmemF64 = 1024 + kDg * kBDig + kBLead + kABufs * kADig + 6144;
-// Outputs whose sum of leading magnitudes is below this take plain products: 128
-// (|a_0| of a power of two) times 40, the smallest E5M2 number above 32 = |b_0| of an
-// entry a binade below its vector's largest.
-constexpr float kLeadMin = 5120.0f;
+// Outputs whose sum of leading magnitudes is below this take plain products.  For rows
+// with one entry: 128 (|a_0| of a power of two) times 40, the smallest E5M2 number above
+// 32 = |b_0| of an entry a binade below its vector's largest.
+constexpr float kLeadMin = 2560.0f, kLeadMinOne = 5120.0f;
 // Magnitude (E5M2, 2^8) that stands for every entry of a zero row, whose outputs are 0
 // unless the vector has no digits.
 constexpr uint32_t kLeadZero = 0x5c;
@@ -102,7 +110,7 @@ struct F64Params {
   double* Y;
   const double* F;      // the factor itself (plain products)
   const uint16_t* img;  // [nchunks][kchunks][digit][k block][128][64], swizzled rows
-  const int* fexp;      // [nchunks][kchunks][128]
+  const int* fexp;      // [nchunks][kchunks][128]: 2 Ef, + 1 for a row with one entry
   int64_t f_i, f_j;     // element strides of F
   int64_t size_in, size_out;
   int rest, tiles_m, ntiles, n_in, n_out, nchunks, kchunks;
@@ -225,58 +233,42 @@ __device__ __forceinline__ bool far_key(int key) {
   return key != 0 && (!has_digits(key) || abs((key >> 20) - 1023) > kFarExp);
 }
 
-// y += alpha f . x over the k chunk [k0, k1) for the columns (vectors) of one mask:
-// column c at x + c and y + c n_out.  Four columns at a time share the loads of f and are
-// a chain each; fewer take four chains each.
+// y += alpha f . x (y = of a single step without old values) over the k chunk [k0, k1)
+// for the columns (vectors) of one mask: column c at x + c and y + c n_out.  Four columns
+// at a time share the loads of f and are a chain each.
 __device__ __forceinline__ void plain_columns(const F64Params& p, uint32_t mask, int k0, int k1,
                                               const double* f, const double* x, double* y) {
   while (mask != 0) {
     int c[4];
-    const bool four = __popc(mask) >= 4;
+    const int nc = min(4, __popc(mask));
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      c[q] = q == 0 || four ? __ffs(mask) - 1 : 0;
-      if (q == 0 || four) mask &= mask - 1;
+      c[q] = q < nc ? __ffs(mask) - 1 : c[0];
+      if (q < nc) mask &= mask - 1;
     }
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     int k = k0;
-    if (four) {
-      for (; k + 4 <= k1; k += 4) {
-        double fv[4], xv[4][4];
+    for (; k + 4 <= k1; k += 4) {
+      double fv[4], xv[4][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          fv[u] = f[(k + u) * p.f_j];
+      for (int u = 0; u < 4; ++u) {
+        fv[u] = f[(k + u) * p.f_j];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) xv[u][q] = x[(int64_t)(k + u) * p.rest + c[q]];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) a[q] = fma(fv[u], xv[u][q], a[q]);
+        for (int q = 0; q < 4; ++q) xv[u][q] = x[(int64_t)(k + u) * p.rest + c[q]];
       }
-      for (; k < k1; ++k)
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          a[q] = fma(f[k * p.f_j], x[(int64_t)k * p.rest + c[q]], a[q]);
-    } else {
-      for (; k + 8 <= k1; k += 8) {
-        double fv[8], xv[8];
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          fv[u] = f[(k + u) * p.f_j];
-          xv[u] = x[(int64_t)(k + u) * p.rest + c[0]];
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) a[u & 3] = fma(fv[u], xv[u], a[u & 3]);
-      }
-      for (; k < k1; ++k) a[0] = fma(f[k * p.f_j], x[(int64_t)k * p.rest + c[0]], a[0]);
-      a[0] = (a[0] + a[1]) + (a[2] + a[3]);
+        for (int q = 0; q < 4; ++q) a[q] = fma(fv[u], xv[u][q], a[q]);
     }
+    for (; k < k1; ++k)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a[q] = fma(f[k * p.f_j], x[(int64_t)k * p.rest + c[q]], a[q]);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      if (q == 0 || four) {
+      if (q < nc) {
         double* o = y + (int64_t)c[q] * p.n_out;
-        *o = fma(p.alpha, a[q], *o);
+        *o = p.kchunks == 1 && !p.has_beta ? p.alpha * a[q] : fma(p.alpha, a[q], *o);
       }
   }
 }
@@ -301,7 +293,6 @@ __global__ void __launch_bounds__(kKc) k_f64_digits(const double* F, int64_t f_i
   const int emax = mx >> 20;
   const bool dig = has_digits(mx);
   const int64_t blk = (int64_t)nc * kchunks + kc;
-  if (k == 0) fexp[blk * kOut + row] = dig ? (mx ? emax - 1023 : 0) : kPlain;
   const unsigned long long u =
       dig && mx ? fixed_digits<3>((unsigned long long)__double_as_longlong(x), emax) : kZeroDigits;
   // digit t: k block (k / 64), row, 16-byte chunk (k / 8) mod 8 swizzled by the row
@@ -309,6 +300,15 @@ __global__ void __launch_bounds__(kKc) k_f64_digits(const double* F, int64_t f_i
                 ((((k >> 3) & 7) ^ (row & 7)) << 3) + (k & 7);
   constexpr size_t st = kADig / 2;
   const uint32_t lead = digit_pair<0>(u, u);
+  // entries of the row with a leading magnitude: one alone takes the strict threshold
+  int cnt = __popc(__ballot_sync(0xffffffffu, (lead & 0x7fffu) != 0));
+  __syncthreads();  // smax is no longer read
+  if ((k & 31) == 0) smax[k >> 5] = cnt;
+  __syncthreads();
+  if (k == 0) {
+    cnt = smax[0] + smax[1] + smax[2] + smax[3];
+    fexp[blk * kOut + row] = (dig ? (mx ? emax - 1023 : 0) : kPlain) * 2 + (cnt <= 1);
+  }
   p[0 * st] = (uint16_t)lead;
   // the leading magnitude: 16-byte chunk k / 16 of the row, swizzled likewise
   reinterpret_cast<unsigned char*>(img + blk * (kABlk / 2))[kDg * kADig + row * kKc +
@@ -408,7 +408,8 @@ __device__ __forceinline__ void put_lead(unsigned char* bdig, unsigned char* ble
 }
 
 // Which of this thread's 32 outputs have too small a sum of leading magnitudes.
-__device__ __forceinline__ uint32_t low_outputs(uint32_t taddr) {
+__device__ __forceinline__ uint32_t low_outputs(uint32_t taddr, bool one) {
+  const float least = one ? kLeadMinOne : kLeadMin;
   uint32_t v[32];
   tmem_ld32(taddr + kDg * kVec, v);
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -416,9 +417,9 @@ __device__ __forceinline__ uint32_t low_outputs(uint32_t taddr) {
 #pragma unroll
   for (int e = 1; e < 32; ++e) mn = fminf(mn, __uint_as_float(v[e]));
   uint32_t low = 0;
-  if (__any_sync(0xffffffffu, mn < kLeadMin)) {
+  if (__any_sync(0xffffffffu, mn < least)) {
 #pragma unroll
-    for (int e = 0; e < 32; ++e) low |= (__uint_as_float(v[e]) < kLeadMin ? 1u : 0u) << e;
+    for (int e = 0; e < 32; ++e) low |= (__uint_as_float(v[e]) < least ? 1u : 0u) << e;
   }
   return low;
 }
@@ -445,7 +446,9 @@ __device__ __forceinline__ void issue_group(uint32_t tmem, uint64_t ad, uint64_t
   }
 }
 
-template <class Src>
+// LOW: low outputs are expected (short factor rows), so that a thread with some still
+// takes the fast drain; its registers cost that 3 to 20 % where there are none.
+template <class Src, bool LOW>
 __global__ void __launch_bounds__(kThreadsF64, 1)
     k_kron_f64_tc(const __grid_constant__ Src src, const F64Launch L) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -731,13 +734,13 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
       const int par = st & 1;
       const int nc = lt % p.nchunks;
       // the factor row's exponent, ahead of its use in the store
-      const int ef = __ldg(&p.fexp[((int64_t)nc * p.kchunks + kc) * kOut + orow]);
+      const int ef2 = __ldg(&p.fexp[((int64_t)nc * p.kchunks + kc) * kOut + orow]);
 #define COLA_DIGIT(S)                                                      \
   if (ok) ok = mbar_wait(&dfull[S], (uint32_t)par, abort_flag, L.err);     \
   ok = __all_sync(0xffffffffu, ok);                                        \
   tc_fence_after();                                                        \
   if (ok) {                                                                \
-    if constexpr (S == 0) clow[tid - 32 * kConvWarps] = low_outputs(taddr); \
+    if constexpr (S == 0) clow[tid - 32 * kConvWarps] = low_outputs(taddr, ef2 & 1); \
     fold<S>(taddr, acc);                                                   \
   }
       COLA_DIGIT(0)
@@ -761,12 +764,22 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
         double* y = p.Y + cur.r * p.size_out + (int64_t)(cur.m0 + oc0) * p.n_out + i;
         const int* keys = ckey + par * kVec + oc0;
         uint32_t low = clow[tid - 32 * kConvWarps];  // outputs that take plain products
+        const int ef = ef2 >> 1;
         const bool near = abs(ef) <= kFarExp && !(cfar[par * 2] | cfar[par * 2 + 1]);
         const int e0 = ef - 53 - 1023;
         // Y's old values join with beta (first k chunk) or 1 (later chunks)
         const bool old = kc > 0 || p.has_beta;
         const double bo = kc > 0 ? 1.0 : p.beta;
-        if (near && low == 0 && cnt == 32) {  // no branch per output
+        auto leave_out = [&](uint32_t mask) {
+          uint32_t* e = L.low + 3 * ((int64_t)blockIdx.x * L.low_cap + atomicAdd(nlow, 1));
+          e[0] = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x * (32 * kDrainWarps) +
+                            tid - 32 * kConvWarps);
+          e[1] = (uint32_t)kc;
+          e[2] = mask;
+        };
+        // LOW: where nothing is added to, the plain products write over their outputs
+        const bool over = LOW && p.kchunks == 1 && !p.has_beta;
+        if (near && (low == 0 || over) && cnt == 32) {  // no branch per output
 #pragma unroll
           for (int g = 0; g < 32; g += 4) {
             double v[4];
@@ -781,6 +794,12 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
               if (old) w = fma(bo, v[c], w);
               y[(g + c) * p.n_out] = w;
             }
+          }
+          if (LOW && low != 0) {
+#pragma unroll 1
+            for (int c = 0; c < 32; ++c)
+              if (keys[c] == 0) low &= ~(1u << c);  // a zero vector's are exact
+            if (low != 0) leave_out(low);
           }
         } else {
           if (cnt < 32) low &= (1u << cnt) - 1;
@@ -808,13 +827,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
             *y = v;
             y += p.n_out;
           }
-          if (low != 0) {
-            uint32_t* e = L.low + 3 * ((int64_t)blockIdx.x * L.low_cap + atomicAdd(nlow, 1));
-            e[0] = (uint32_t)((tile - (int)blockIdx.x) / (int)gridDim.x * (32 * kDrainWarps) +
-                              tid - 32 * kConvWarps);
-            e[1] = (uint32_t)kc;
-            e[2] = low;
-          }
+          if (low != 0) leave_out(low);
         }
       }
       __syncwarp();
@@ -834,21 +847,24 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
                  "r"(512)
                  : "memory");
   }
-  // The outputs left out above, on the FP64 units (their rate bounds it: a tile
-  // whose outputs are all plain takes 260 us).  Y is this CTA's own.
-  // One k chunk after the other, as an output may be left out of several.
+  // The outputs left out above, on the FP64 units (their rate bounds it: 300 us a
+  // tile whose outputs are all plain).  Y is this CTA's own.
+  // One k chunk after the other, as an output may be left out of several; eight columns
+  // of an entry to a thread, so that a few entries still reach every warp.
   const int entries = *abort_flag ? 0 : *nlow;
   for (int kc = 0; kc < (entries ? L.kmax : 0); ++kc) {
-    for (int n = tid; n < entries; n += kThreadsF64) {
+    for (int64_t u = tid; u < 4 * (int64_t)entries; u += kThreadsF64) {
+      const int n = (int)(u % entries);
       const uint32_t* e = L.low + 3 * ((int64_t)blockIdx.x * L.low_cap + n);
-      if (e[1] != (uint32_t)kc) continue;
+      const uint32_t mask = e[2] & 0xffu << (8 * (int)(u / entries));
+      if (e[1] != (uint32_t)kc || mask == 0) continue;
       const int thr = e[0] % (32 * kDrainWarps);
       int lt;
       const F64Params& p = src.get(
           (int)blockIdx.x + (int)(e[0] / (32 * kDrainWarps)) * (int)gridDim.x, lt);
       const F64Step cur = step_of(p, lt, kc);
       const int i = cur.nc * kOut + thr % kOut, m = cur.m0 + thr / kOut * 32;
-      plain_columns(p, e[2], kc * kKc, min(p.n_in, (kc + 1) * kKc), p.F + i * p.f_i,
+      plain_columns(p, mask, kc * kKc, min(p.n_in, (kc + 1) * kKc), p.F + i * p.f_i,
                     p.X + cur.r * p.size_in + m,
                     p.Y + cur.r * p.size_out + (int64_t)m * p.n_out + i);
     }
@@ -873,16 +889,16 @@ static bool f64_low_list(Ctx* c, int ntiles, int kchunks, F64Launch* L) {
   return L->low != nullptr;
 }
 
-template <class Src>
+template <class Src, bool LOW>
 static void f64_launch(Ctx* c, const Src& src, int ntiles, F64Launch L) {
   L.err = tc_errflag(c);
   if (c->tc_stall_ns > 0 && !c->capturing) {
     L.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
     c->tc_stall_ns = 0;
   }
-  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemF64));
-  k_kron_f64_tc<Src><<<std::min(ntiles, c->num_sms), kThreadsF64, kSmemF64, c->s>>>(src, L);
+  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc<Src, LOW>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemF64));
+  k_kron_f64_tc<Src, LOW><<<std::min(ntiles, c->num_sms), kThreadsF64, kSmemF64, c->s>>>(src, L);
   c->count_launch();
   c->f64_tc_used = true;
   COLA_CUDA(cudaGetLastError());
@@ -951,7 +967,7 @@ bool f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
                             cudaMemcpyHostToDevice, c->s));
   COLA_CUDA(cudaMemcpyAsync((void*)src.first, first.data(), 4 * (size_t)np,
                             cudaMemcpyHostToDevice, c->s));
-  f64_launch(c, src, nt, L);
+  f64_launch<F64Tab, false>(c, src, nt, L);
   COLA_CUDA(cudaStreamSynchronize(c->s));  // the host tables go out of scope
   return true;
 }
@@ -1000,7 +1016,12 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.beta = beta;
   p.has_alpha = alpha != 1.0;
   p.has_beta = beta != 0.0;
-  f64_launch(c, F64One{p}, p.ntiles, L);
+  // an RBF factor of lengthscale 0.05 on n uniform points leaves 3 % of its outputs low
+  // at n = 32 and 0.1 % at n = 64
+  if (n_in <= 64)
+    f64_launch<F64One, true>(c, F64One{p}, p.ntiles, L);
+  else
+    f64_launch<F64One, false>(c, F64One{p}, p.ntiles, L);
   return true;
 }
 

@@ -3,11 +3,11 @@ a mode step is within a bound of its own sum |f| |x|, whatever the other entries
 of its factor row and vector are.
 
 Bound of one mode step with K contracted entries.  An output keeps its digit
-product only where the sum of leading magnitudes is at least 5120.  A leading
+product only where the sum of leading magnitudes is at least 2560.  A leading
 magnitude is at most twice |f| 2^(7 - Ef) or |x| 2^(6 - Ex), so there sum |f| |x| >=
-5120 / 4 2^-13 2^(Ef + Ex) > 2^-3 2^(Ef + Ex).  Dropped digit pairs (6 2^-55), x kept
+2560 / 4 2^-13 2^(Ef + Ex) = 2^-3.68 2^(Ef + Ex).  Dropped digit pairs (6 2^-55), x kept
 to 2^-55 and f to 2^-56 of 2^Ex and 2^Ef are at most 1.14 2^-52 K 2^(Ef + Ex), hence at
-most 1.14 2^-49 K sum |f| |x|; with the roundings, 2^-48 K sum |f| |x|.  Plain FP64
+most 0.92 2^-48 K sum |f| |x|; with the roundings, 2^-48 K sum |f| |x|.  Plain FP64
 products stay within 2^-53 K sum |f| |x|.  Contributions of a later k chunk may
 also be hidden by the sum so far: 1.14 2^-52 K 2^-4 of it, and that sum is at most
 sum |f| |x| of its chunks."""
@@ -48,8 +48,8 @@ def _rbf(r, n, ell, ordered=False):
 
 def test_identity_factors_return_graded_vectors():
     """Entries of one fibre 18 and 100 orders apart come back exactly: 0 and 1 times
-    them are exact, in FP64 multiply-adds and in digits, which an output of an identity
-    factor takes only from an entry within a binade of its vector's largest."""
+    them are exact, in FP64 multiply-adds and in digits, which an output of a row with
+    one entry takes only from an entry within a binade of its vector's largest."""
     r = np.random.default_rng(1)
     X = r.standard_normal((8, 128 * 128))
     X[:, ::3] *= 1e-18
@@ -86,3 +86,22 @@ def test_outputs_are_accurate_entry_by_entry(sides, R, kind):
         X = r.standard_normal((R, N))
         X[0, : N // 2] = 0.0
     _check(F, X)
+
+
+@pytest.mark.parametrize("n,R", [(128, 6), (64, 64), (200, 5)])
+def test_residuals_of_identity_factors_are_exact(n, R):
+    """Old values and a factor of -1: b - A x of a solve that starts from its solution,
+    with entries of one fibre 18 orders apart, is 0 (the products are exact)."""
+    import paper_2309_03060_gb300 as cola
+    r = np.random.default_rng(n)
+    X = r.standard_normal((R, n * n))
+    X[:, ::3] *= 1e-18
+    X[1, : n // 2] = 0.0
+    ctx = cola.cola_create(0)
+    eye = torch.eye(n, dtype=torch.float64, device="cuda")
+    op = cola.cola_linop_kron(ctx, *[cola.cola_linop_dense(ctx, eye) for _ in range(2)]).set_spd()
+    B = torch.tensor(X, device="cuda")
+    opts = cola.cola_cg_opts_default(precision=cola.PREC_MIXED, refine=1, tol=1e-10, maxiter=0)
+    Y, info, st = cola.cola_cg_solve(ctx, op, B, opts, X0=B)
+    assert st == 0 and [i["rel_residual"] for i in info] == [0.0] * R
+    assert torch.equal(Y, B)

@@ -568,10 +568,12 @@ cola_status batched_cg_fast(Ctx* c, int32_t nsys, const cola_linop* const* ops,
 
   // The FP64 residual products run as digit products on the tensor cores
   // (kron_f64.cu) where that is faster: steps of 64 vectors x 128 outputs x 128 k
-  // spread over the SMs at 15 us each plus 40 us of launches and fill, against
-  // 0.55e6 multiply-adds per us in 32 x 32 tiles on the FP64 units (the rule of a
-  // single product, f64_tc_pays, summed over the problems).  Measured on 64 systems
-  // with sides 16 .. 256: 153 us a product against 788 us.
+  // spread over the SMs at 15 us each plus 40 us of launches and fill, against 20 us plus
+  // 0.55e6 multiply-adds per us in 32 x 32 tiles on the FP64 units.  A fit of its own:
+  // a step costs more than the 10.5 us of a single product (f64_tc_pays) since its
+  // fields come from a table, and whole waves do not count where the tiles of many
+  // problems share a launch.  Measured on 64 systems with sides 16 .. 256: 153 us a
+  // product against 788 us.
   auto f64_gain = [&](auto&& counted) {
     double steps = 0.0, fma = 0.0;
     bool fits = true;

@@ -140,10 +140,12 @@ __global__ void __launch_bounds__(256) k_gemm(GemmP<T> g, int64_t batch0) {
 // fma.rn.f32x2 does two multiply-adds (half the issue slots; same rounding).
 // The next k tile's loads are held in registers while the current one is
 // multiplied out of the other shared-memory buffer.  TN follows the factor's
-// side, so that a side of 97 runs 112 wide instead of 128.  Bound by the FP32
-// pipe and the shared-memory reads: 97 x 120 x 101, 5 vectors, 135 us for the
-// three modes (28 TFLOP/s of 80.5; 144 us with one 4-byte load per column) against
-// 288 us in the generic 128 x 128 tiles that unaligned sides took before.
+// side, so that a side of 97 runs 112 wide instead of 128.  97 x 120 x 101, 5 vectors:
+// 135 us for the three modes (28 TFLOP/s of 80.5; 144 us with one 4-byte load per column)
+// against 288 us in the generic 128 x 128 tiles that unaligned sides took before.  Not at
+// a unit's limit: 385 to 475 equal blocks on 304 slots (1.3 to 1.6 waves), the FP32 pipe
+// active half of the time while they run, and the diagonal's loads in the last mode's
+// epilogue (a third active there).
 constexpr int kMfBM = 128, kMfBK = 16;
 
 __device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a,

@@ -1016,9 +1016,11 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.beta = beta;
   p.has_alpha = alpha != 1.0;
   p.has_beta = beta != 0.0;
-  // an RBF factor of lengthscale 0.05 on n uniform points leaves 3 % of its outputs low
-  // at n = 32 and 0.1 % at n = 64
-  if (n_in <= 64)
+  // RBF factors on n uniform points leave 0.2 % (lengthscale 0.05) and 0.01 % (0.1) of
+  // their outputs low at n = 32, more on draws with lone points, but 0.005 % and none at
+  // n = 48: from there the fast drain's registers count for more (34 x 128 x 82, 14
+  // vectors, lengthscale 0.22: 309 -> 336 us with LOW in the first mode alone)
+  if (n_in <= 48)
     f64_launch<F64One, true>(c, F64One{p}, p.ntiles, L);
   else
     f64_launch<F64One, false>(c, F64One{p}, p.ntiles, L);

@@ -1311,7 +1311,7 @@ static ModeF32 mode_f32_kernel(int tn) {
 // 12 us for the digit images and a pipeline's fill plus 10.5 us per step (64
 // vectors x 128 outputs x 128 k) a CTA runs one after the other, against 6 us
 // plus 0.55e6 multiply-adds per us in 32 x 32 tiles.  Measured, us a step: 128^3 x
-// 16 264 against 6970; 64^2 x 64 21 against 37; 128^2 x 4 23 against 20.
+// 16 270 against 6970; 64^2 x 64 21 against 37; 128^2 x 4 23 against 20.
 static bool f64_tc_pays(const Ctx* c, int64_t M, int64_t N, int64_t K, int64_t batch) {
   const double tiles = (double)((M + 63) / 64) * (double)((N + 127) / 128) * (double)batch;
   const double waves = std::ceil(tiles / c->num_sms);

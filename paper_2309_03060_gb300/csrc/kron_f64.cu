@@ -29,10 +29,10 @@
 // 32 .. 200: 0.6 .. 5.4, against 3.3 .. 9.9 in FP64 multiply-adds; graded vectors 20
 // against 20, identity 0 against 0, unit vectors 1.6 against 0.  What it costs: nothing
 // where no output is low, the rate of the FP64 units where most are (identity 128^3 x 4:
-// 6.1 ms for the three steps, 5.25 ms in 32 x 32 tiles there; columns of a 128 x 128 RBF
-// product, 64 of them: 0.33 against 0.47 ms), and on short RBF factors of a small
+// 5.8 ms for the three steps, 5.25 ms in 32 x 32 tiles there; columns of a 128 x 128 RBF
+// product, 64 of them: 0.30 against 0.47 ms), and on short RBF factors of a small
 // lengthscale, some of whose points have no neighbour, part of the gain: sides 32, 48,
-// lengthscale 0.05, 16 vectors 134, 205 us against 87, 140 without it and 123, 625 on the
+// lengthscale 0.05, 16 vectors 123, 184 us against 87, 140 without it and 123, 625 on the
 // FP64 units.
 //
 // Why: this GPU's FP64 units do 2 multiply-adds per clock and SM (1.2 TFLOP/s),
@@ -58,15 +58,15 @@
 //               D_s is drained and digit 6 - s refilled for the next step while
 //               the later groups run, and only D_6 and digit 0 are left when the
 //               MMAs of a step end
-// Measured (128^3 x 16, one mode step, 268 MB in and out): 265 us against 6.97 ms
+// Measured (128^3 x 16, one mode step, 268 MB in and out): 270 us against 6.97 ms
 // on the FP64 units.  What bounds it: the chain of conversion, MMAs and drain of a
 // step, each waiting for the one before with 18 warps on the SM: the integer pipe (8192
 // entries converted, 8192 outputs combined per step) is active 0.58 of the time, the
 // tensor-core pipe (224 MMAs of 128 x 64 x 16 per step) 0.61, issue slots 0.50;
 // converting and draining in separate warps, both beside the MMAs, took it from 395 us,
 // no FP64 conversion per output from 450 us, and issuing from a converged warp (uniform
-// descriptors) from 520 us.  18 warps hold a thread to 96 registers (56 bytes of spills;
-// 260 in the variants for short factors and for a table of problems).
+// descriptors) from 520 us.  18 warps hold a thread to 96 registers (72 bytes of spills;
+// 280 in the variant with a table of problems).
 // Accumulators: D_0 .. D_6 and the magnitudes', 64 FP32 columns each of tensor memory
 // (all 512).  Every mbarrier wait gives up after ~2 s and raises the error flag.
 #include <cuda_fp16.h>
@@ -100,8 +100,8 @@ constexpr size_t kSmemF64 = 1024 + kDg * kBDig + kBLead + kABufs * kADig + 6144;
 // with one entry: 128 (|a_0| of a power of two) times 40, the smallest E5M2 number above
 // 32 = |b_0| of an entry a binade below its vector's largest.
 constexpr float kLeadMin = 2560.0f, kLeadMinOne = 5120.0f;
-// Magnitude (E5M2, 2^8) that stands for every entry of a zero row, whose outputs are 0
-// unless the vector has no digits.
+// Magnitude (E5M2, 2^8) that stands for every entry of a zero row or vector, whose outputs
+// are exact (0, or without digits on the other side).
 constexpr uint32_t kLeadZero = 0x5c;
 constexpr int kPlain = 1 << 20;  // exponent mark of a factor row that takes plain products
 
@@ -386,10 +386,11 @@ __device__ __forceinline__ void put_digit(unsigned char* bdig, const unsigned lo
 
 // put_digit<0> and this thread's leading magnitudes, |digit 0| truncated to E5M2 (the
 // upper byte of its FP16 form), up to kpad rounded to the 32 k of an 8-bit MMA
-// (entries past n_in are zeros).
+// (entries past n_in are zeros); keys: the four magnitude keys of the vector.
 __device__ __forceinline__ void put_lead(unsigned char* bdig, unsigned char* blead,
                                          const unsigned long long (&u)[32], int n, int oct,
-                                         int kpad) {
+                                         int kpad, const int* keys) {
+  const bool zero = (keys[0] | keys[kVec] | keys[2 * kVec] | keys[3 * kVec]) == 0;
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
     if (oct * 8 + h * 32 >= (kpad + 31) / 32 * 32) continue;
@@ -400,8 +401,9 @@ __device__ __forceinline__ void put_lead(unsigned char* bdig, unsigned char* ble
     w.w = digit_pair<0>(u[8 * h + 6], u[8 * h + 7]);
     const int ch = (oct + 4 * (h & 1)) ^ (n & 7);
     *reinterpret_cast<uint4*>(bdig + (h >> 1) * (kBDig / 2) + n * 128 + ch * 16) = w;
-    const uint2 m = make_uint2(__byte_perm(w.x, w.y, 0x7531) & 0x7f7f7f7fu,
-                               __byte_perm(w.z, w.w, 0x7531) & 0x7f7f7f7fu);
+    uint2 m = make_uint2(__byte_perm(w.x, w.y, 0x7531) & 0x7f7f7f7fu,
+                         __byte_perm(w.z, w.w, 0x7531) & 0x7f7f7f7fu);
+    if (zero) m = make_uint2(kLeadZero * 0x01010101u, kLeadZero * 0x01010101u);
     *reinterpret_cast<uint2*>(blead + n * kKc + ((((oct >> 1) + 2 * h) ^ (n & 7)) << 4) +
                               (oct & 1) * 8) = m;
   }
@@ -446,9 +448,7 @@ __device__ __forceinline__ void issue_group(uint32_t tmem, uint64_t ad, uint64_t
   }
 }
 
-// LOW: low outputs are expected (short factor rows), so that a thread with some still
-// takes the fast drain; its registers cost that 3 to 20 % where there are none.
-template <class Src, bool LOW>
+template <class Src>
 __global__ void __launch_bounds__(kThreadsF64, 1)
     k_kron_f64_tc(const __grid_constant__ Src src, const F64Launch L) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
   if constexpr (S < 6)                                                     \
     put_digit<6 - S>(bdig, u, n, oct, kpad);                               \
   else                                                                     \
-    put_lead(bdig, blead, u, n, oct, kpad);
+    put_lead(bdig, blead, u, n, oct, kpad, cmax + par * 4 * kVec + n);
       COLA_DIGIT(0)
       COLA_DIGIT(1)
       COLA_DIGIT(2)
@@ -777,8 +777,8 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
           e[1] = (uint32_t)kc;
           e[2] = mask;
         };
-        // LOW: where nothing is added to, the plain products write over their outputs
-        const bool over = LOW && p.kchunks == 1 && !p.has_beta;
+        // where nothing is added to, the plain products write over their outputs
+        const bool over = p.kchunks == 1 && !p.has_beta;
         if (near && (low == 0 || over) && cnt == 32) {  // no branch per output
 #pragma unroll
           for (int g = 0; g < 32; g += 4) {
@@ -795,12 +795,7 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
               y[(g + c) * p.n_out] = w;
             }
           }
-          if (LOW && low != 0) {
-#pragma unroll 1
-            for (int c = 0; c < 32; ++c)
-              if (keys[c] == 0) low &= ~(1u << c);  // a zero vector's are exact
-            if (low != 0) leave_out(low);
-          }
+          if (low != 0) leave_out(low);
         } else {
           if (cnt < 32) low &= (1u << cnt) - 1;
 #pragma unroll 1
@@ -814,11 +809,11 @@ __global__ void __launch_bounds__(kThreadsF64, 1)
             if (abs(ef) > kFarExp || far_key(key)) {  // out of scaled_double's range
               low |= 1u << c;
             } else if (low >> c & 1u) {
-              // too small a sum of leading magnitudes, except where the digits are exact (a
-              // zero vector) and where their error, below 2^-51 K 2^(Ef + Ex), is hidden by
-              // the rounding of a sum so far of at least 2^kHidden of that binade
-              if (key == 0 || (kc > 0 && fabs(yo) >= fabs(p.alpha) *
-                                             __hiloint2double((1023 + 53 + kHidden + e) << 20, 0)))
+              // too small a sum of leading magnitudes, except where the digits' error, below
+              // 2^-51 K 2^(Ef + Ex), is hidden by the rounding of a sum so far of at least
+              // 2^kHidden of that binade
+              if (kc > 0 && fabs(yo) >= fabs(p.alpha) *
+                                            __hiloint2double((1023 + 53 + kHidden + e) << 20, 0))
                 low ^= 1u << c;
             }
             double v = scaled_double(low >> c & 1u ? 0ll : ac, e);
@@ -889,16 +884,16 @@ static bool f64_low_list(Ctx* c, int ntiles, int kchunks, F64Launch* L) {
   return L->low != nullptr;
 }
 
-template <class Src, bool LOW>
+template <class Src>
 static void f64_launch(Ctx* c, const Src& src, int ntiles, F64Launch L) {
   L.err = tc_errflag(c);
   if (c->tc_stall_ns > 0 && !c->capturing) {
     L.stall_ns = (uint64_t)c->tc_stall_ns;  // armed once by cola_test_stall_next_launch
     c->tc_stall_ns = 0;
   }
-  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc<Src, LOW>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemF64));
-  k_kron_f64_tc<Src, LOW><<<std::min(ntiles, c->num_sms), kThreadsF64, kSmemF64, c->s>>>(src, L);
+  COLA_CUDA(cudaFuncSetAttribute(k_kron_f64_tc<Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemF64));
+  k_kron_f64_tc<Src><<<std::min(ntiles, c->num_sms), kThreadsF64, kSmemF64, c->s>>>(src, L);
   c->count_launch();
   c->f64_tc_used = true;
   COLA_CUDA(cudaGetLastError());
@@ -967,7 +962,7 @@ bool f64_tc_batch(Ctx* c, const std::vector<F64Batch>& probs, const char* tag) {
                             cudaMemcpyHostToDevice, c->s));
   COLA_CUDA(cudaMemcpyAsync((void*)src.first, first.data(), 4 * (size_t)np,
                             cudaMemcpyHostToDevice, c->s));
-  f64_launch<F64Tab, false>(c, src, nt, L);
+  f64_launch(c, src, nt, L);
   COLA_CUDA(cudaStreamSynchronize(c->s));  // the host tables go out of scope
   return true;
 }
@@ -1016,14 +1011,7 @@ bool f64_tc_mode_step(Ctx* c, int64_t rest, int n_out, int n_in, double alpha, c
   p.beta = beta;
   p.has_alpha = alpha != 1.0;
   p.has_beta = beta != 0.0;
-  // RBF factors on n uniform points leave 0.2 % (lengthscale 0.05) and 0.01 % (0.1) of
-  // their outputs low at n = 32, more on draws with lone points, but 0.005 % and none at
-  // n = 48: from there the fast drain's registers count for more (34 x 128 x 82, 14
-  // vectors, lengthscale 0.22: 309 -> 336 us with LOW in the first mode alone)
-  if (n_in <= 48)
-    f64_launch<F64One, true>(c, F64One{p}, p.ntiles, L);
-  else
-    f64_launch<F64One, false>(c, F64One{p}, p.ntiles, L);
+  f64_launch(c, F64One{p}, p.ntiles, L);
   return true;
 }
 
